@@ -1,0 +1,567 @@
+// Dense-tile SpMM on the tensor cores for BF16 matrices of a few percent of entries and more.
+//
+// At 90% sparsity a row split gathers one B row (512 bytes at N = 256) per stored entry from
+// L2, 13.7 GB on 16,384^2, while the whole dense product is 137 GFLOP, 73 us at the measured
+// cuBLAS rate.  So A is expanded: a CTA takes 128 rows of A and all of (up to 256 columns of)
+// B, walks A's columns 64 at a time, scatters a 128 x 64 tile's entries into a zeroed tile in
+// shared memory (already in the MMA's K-major 128-byte-swizzled image), loads the 64 B rows by
+// TMA and multiplies with tcgen05.mma (M = 128 rows, N = the features, K = 64).
+//
+// The products of BF16 values are exact; the tensor core's accumulation is not rounded to
+// nearest, and its error grows with the number of steps.  So an accumulator in TMEM runs over
+// 512 columns only, and the worker warps add it to FP32 sums in registers, two accumulators
+// alternating.  Error against 64 bits on 16,384^2 at 90%, uniform: 1.53e-7 with 256 columns per
+// accumulator (where the register sums' rounding dominates), 1.28e-7 with 512, 1.50e-7 with
+// 1,024; the CSR kernel has 2.0e-7 (N = 256), the 16 x 8 blocks over all columns 9.7e-7.
+//
+// The expanded zeros meet B's values: an infinity or NaN in any B row makes NaN in every row
+// of C.  Every accumulated value is tested at the end, and a block with one that is not finite
+// is computed again from the CSR arrays on the CUDA cores, where only stored entries count.
+#include <mutex>
+
+#include "spmm_kernels.cuh"
+#include "tc_dense.cuh"
+
+namespace gbsp {
+
+EncodeTiledFn encode_fn() {
+    static EncodeTiledFn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiledFn>(p);
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
+
+namespace dense {
+namespace {
+
+using namespace gbsp::tc;
+
+// ---- regrouping -----------------------------------------------------------------------------
+
+constexpr int kBinThreads = 1024;
+constexpr int kMaxTiles = 8 * 1024;   // one shared-memory counter per tile of a row block
+
+// Runs f(column, run length, first lane of the run, lane of this entry) over 32 entries of a row
+// at a time; a run is a maximal stretch of entries in one tile (a run cut by a chunk's end is
+// two runs).  Returns false when the columns are not strictly increasing in [0, K).
+template <class F>
+__device__ __forceinline__ bool for_runs(const int32_t *colidx, int64_t p0, int64_t p1, int K, int lane, F f) {
+    bool good = true;
+    for (int64_t base = p0; base < p1; base += 32) {
+        const int64_t p = base + lane;
+        const bool in = p < p1;
+        const int c = in ? __ldg(colidx + p) : 0x7fffffff;
+        int prev = __shfl_up_sync(FULL, c, 1);
+        if (lane == 0) prev = base > p0 ? __ldg(colidx + base - 1) : -1;
+        if (in && (c <= prev || c < 0 || c >= K)) good = false;
+        const unsigned heads =
+            __ballot_sync(FULL, in && (lane == 0 || (c / kCols) != (prev / kCols)));
+        const int cnt = p1 - base < 32 ? (int)(p1 - base) : 32;
+        const unsigned upto = heads & (FULL >> (31 - lane));
+        const int first = upto ? 31 - __clz(upto) : 0;
+        const unsigned after = lane == 31 ? 0u : heads & (FULL << (lane + 1));
+        const int end = after ? __ffs(after) - 1 : cnt;
+        f(p, in && c >= 0 && c < K, c, first, end - first);
+    }
+    return __all_sync(FULL, good);
+}
+
+// One CTA per block of 128 rows: counts the entries per tile, turns the counts into offsets and
+// writes each entry's packed word at the tile's cursor (the order inside a tile is free: every
+// entry has its own place in the tile).
+__global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restrict__ rowptr,
+                                                          const int32_t *__restrict__ colidx,
+                                                          const uint16_t *__restrict__ vals, int M, int K, int nkt,
+                                                          Tiles t) {
+    extern __shared__ int32_t cnt[];  // nkt counters, then cursors
+    __shared__ int32_t warp_sum[32];
+    __shared__ int32_t carry;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int b = blockIdx.x, r0 = b * kRows, r1 = min(r0 + kRows, M);
+    for (int i = tid; i < nkt; i += kBinThreads) cnt[i] = 0;
+    if (tid == 0) carry = 0;
+    __syncthreads();
+    bool good = true;
+    for (int r = r0 + warp; r < r1; r += kBinThreads / 32)
+        good &= for_runs(colidx, __ldg(rowptr + r), __ldg(rowptr + r + 1), K, lane,
+                         [&](int64_t, bool in, int c, int first, int len) {
+                             if (in && first == lane) atomicAdd(&cnt[c / kCols], len);
+                         });
+    const bool bad = !__syncthreads_and(good);
+    const int32_t start = __ldg(rowptr + r0);
+    int32_t *tp = t.tptr + (int64_t)b * (nkt + 1);
+    for (int base = 0; base < nkt; base += kBinThreads) {
+        const int i = base + tid;
+        const int v = i < nkt ? cnt[i] : 0;
+        int x = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        int before = carry;
+        for (int w = 0; w < warp; ++w) before += warp_sum[w];
+        if (i < nkt) {
+            cnt[i] = start + before + x - v;
+            tp[i] = start + before + x - v;
+        }
+        __syncthreads();
+        if (tid == kBinThreads - 1) carry = before + x;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        tp[nkt] = start + carry;
+        t.bad[b] = bad ? 1 : 0;
+    }
+    if (bad) return;
+    for (int r = r0 + warp; r < r1; r += kBinThreads / 32)
+        for_runs(colidx, __ldg(rowptr + r), __ldg(rowptr + r + 1), K, lane,
+                 [&](int64_t p, bool in, int c, int first, int len) {
+                     int at = 0;
+                     if (in && first == lane) at = atomicAdd(&cnt[c / kCols], len);
+                     at = __shfl_sync(FULL, at, first) + lane - first;
+                     if (in) {
+                         const int rr = r - r0, cc = c % kCols;
+                         const uint32_t off = rr * 128 + (((cc >> 3) ^ (rr & 7)) << 4) + (cc & 7) * 2;
+                         t.ent[at] = ((uint32_t)__ldg(vals + p) << 16) | off;
+                     }
+                 });
+}
+
+// ---- product --------------------------------------------------------------------------------
+
+constexpr int kGroups = 4;                      // groups of four warps that expand tiles and drain accumulators
+constexpr int kWorkers = 4 * kGroups;
+constexpr int kThreads = (kWorkers + 2) * 32;   // + one warp that copies, one that issues MMAs
+constexpr int kATileBytes = kRows * kCols * 2;  // 16 KB
+constexpr int kTurns = 2;                       // turns of all groups per TMEM accumulator
+constexpr int kChunk = kTurns * kGroups;        // its tiles: 512 columns of A
+constexpr int kSlot = 1072;                     // words of an entry slot (any more come from global memory)
+constexpr int kAhead = 3;                       // turns between the L2 prefetch of a tile's entries and their copy
+
+template <int NT>
+struct Shape {
+    static constexpr int BT = kCols * NT * 2;         // bytes of a tile's B rows
+    static constexpr int SB = NT == 256 ? 4 : NT == 128 ? 6 : 8;  // tiles whose B rows are held or on their way
+    static constexpr int R = NT == 256 ? 2 : 3;       // entry slots of a group: one is read, the others on their way
+    static constexpr int SLOTS = R * kGroups;
+    static constexpr int SMEM = kGroups * kATileBytes + SB * BT + SLOTS * (kSlot * 4 + 24) + 1024 + 256;
+};
+
+struct Args {
+    Tiles t;
+    int32_t *marks;  // [feature tile][row block]: 1 where the block is to be computed again
+    float *C;
+    int64_t ldc;
+    int M, N, nkt;
+    int vec;  // floats per store: 8 (32-byte aligned C rows), 4 or 1
+    int *err;
+    int withhold;
+};
+
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Barrier of n threads that returns the conjunction of their votes.
+__device__ __forceinline__ bool bar_all(int id, int n, bool vote) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(id), "r"(n), "r"((uint32_t)vote)
+        : "memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void st_shared_u16(uint32_t addr, uint16_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
+}
+__device__ __forceinline__ void st_shared_zero16(uint32_t addr) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0) : "memory");
+}
+
+// grid (row blocks, feature tiles of NT).  What bounds it at N = 256 is the chain around one of
+// the four expanded tiles (MMAs done, zero, barrier, scatter, MMAs), 0.46 us a tile against
+// 0.34 for the MMAs at cuBLAS's rate.  Sixteen warps expand: a group of four owns an expanded tile
+// and takes every fourth, so its chain has four tiles' time.  Measured on 16,384^2 at 90%, half in
+// dense blocks, N = 256 (the 16 x 8 blocks + residual kernel before: 415 us): 264 us with two
+// groups and entries loaded to registers a tile ahead, 170 with the entries copied to shared
+// memory, 150 with four groups, 124 with the entry loop unpredicated, 119 with the MMAs issued
+// from a uniform loop.
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1) spmm_kernel(const __grid_constant__ CUtensorMap tmB,
+                                                                         const Args a) {
+    using SH = Shape<NT>;
+    constexpr int S = kGroups, R = SH::R, SB = SH::SB, W = NT / kGroups;  // W: columns of the sums that a thread holds
+    const int b = blockIdx.x;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *bring = smem + S * kATileBytes;  // (a group owns one expanded tile, and takes every fourth)
+    uint32_t *ring = reinterpret_cast<uint32_t *>(bring + SB * SH::BT);
+    int4 *hdr = reinterpret_cast<int4 *>(ring + SH::SLOTS * kSlot);  // per slot: words to skip, words, first, last entry
+    uint64_t *full = reinterpret_cast<uint64_t *>(hdr + SH::SLOTS);  // a tile is expanded and its B rows landed
+    uint64_t *empty = full + SB;                                         // ... and its MMAs are done
+    uint64_t *cdone = empty + SB;                                        // an accumulator is complete
+    uint64_t *bfree = cdone + 2;                                         // ... and drained
+    uint64_t *efull = bfree + 2;                                         // a ring slot's entries landed
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(efull + SH::SLOTS);
+    int *failed = reinterpret_cast<int *>(tslot + 1);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (a.t.bad && __ldg(a.t.bad + b)) {  // the block's entries were not regrouped
+        if (tid == 0) a.marks[blockIdx.y * gridDim.x + b] = 1;
+        return;
+    }
+    const int nst = a.nkt, nchunks = (nst + kChunk - 1) / kChunk;
+    const int32_t *tp = a.t.tptr + (int64_t)b * (a.nkt + 1);
+    const int n0 = blockIdx.y * NT;
+
+    if (tid == 0) {
+        for (int s = 0; s < SB; ++s) {
+            mbar_init(&full[s], 1 + 4);
+            mbar_init(&empty[s], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&cdone[i], 1);
+            mbar_init(&bfree[i], kWorkers);
+        }
+        for (int i = 0; i < SH::SLOTS; ++i) mbar_init(&efull[i], 1);
+        *failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+    }
+    if (warp == 0) tmem_alloc(tslot, 2 * NT);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t taddr = *tslot;
+
+    // Sums of the even and of the odd accumulators where the registers allow both, half as many
+    // roundings each (error on 16,384^2 at 95%, N = 128: 1.37e-7 with one sum over accumulators of
+    // 256 columns, 9.0e-8 with two over 512; the CSR kernel has 9.6e-8)
+    constexpr int P = NT == 256 ? 1 : 2;
+    float acc[P][W];
+#pragma unroll
+    for (int k = 0; k < P * W; ++k) acc[k / W][k % W] = 0.f;
+
+    if (warp < kWorkers) {
+        const int g = warp >> 2, t = tid & 127;
+        const uint32_t tlane = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + g * W;
+        const uint32_t at = smem_u32(smem + g * kATileBytes);
+        bool ok = true;
+        int drained = 0;
+        auto drain = [&](int c) {  // adds accumulator c to the sums and frees its buffer
+            const int buf = c & 1;
+            ok = ok && __all_sync(FULL, mbar_wait(&cdone[buf], (c >> 1) & 1));
+            if (!ok) return;
+            fence_after_sync();
+            auto add = [&](float (&sum)[W]) {
+#pragma unroll
+                for (int k = 0; k < W; k += 16) {
+                    float r[16];
+                    tmem_ld16(tlane + buf * NT + k, r);
+#pragma unroll
+                    for (int j = 0; j < 16; j += 2) {
+                        const float2 v =
+                            __fadd2_rn(make_float2(sum[k + j], sum[k + j + 1]), make_float2(r[j], r[j + 1]));
+                        sum[k + j] = v.x;
+                        sum[k + j + 1] = v.y;
+                    }
+                }
+            };
+            if (P == 1 || buf == 0)
+                add(acc[0]);
+            else
+                add(acc[P - 1]);
+            fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bfree[buf]);
+        };
+        // The group's first thread sends for tiles' entries (turn k's go to slot R * g + k % R) once
+        // the whole group is past that slot's previous tile: a bulk copy from the 16-byte boundary
+        // before the first entry.  A copy from HBM takes about a turn (1.6 us), so the entries
+        // are brought to L2 three turns earlier.
+        int sent = g, f0 = 0, f1 = 0, q0 = 0, q1 = 0;
+        auto bounds = [&]() {  // of the next tile to send for and to bring to L2, a turn ahead
+            if (sent < nst) {
+                f0 = __ldg(tp + sent);
+                f1 = __ldg(tp + sent + 1);
+            }
+            const int q = sent + kAhead * kGroups;
+            q0 = q < nst ? __ldg(tp + q) & ~3 : 0;
+            q1 = q < nst ? __ldg(tp + q + 1) : 0;
+        };
+        auto send = [&]() {
+            if (q1 > q0) prefetch_l2(a.t.ent + q0, ((q1 - q0) * 4 + 15) & ~15);
+            const int sl = R * g + sent / kGroups % R, skip = f0 & 3;
+            const int words = min((f1 - f0 + skip + 3) & ~3, kSlot);
+            hdr[sl] = make_int4(skip, f1 > f0 ? min(f1 - f0, kSlot - skip) : 0, f0, f1);
+            if (f1 > f0) {
+                mbar_expect_tx(&efull[sl], words * 4);
+                bulk_load(ring + sl * kSlot, a.t.ent + (f0 - skip), words * 4, &efull[sl]);
+            } else {
+                mbar_arrive(&efull[sl]);
+            }
+            sent += kGroups;
+            bounds();
+        };
+        if (t == 0) {
+            bounds();
+            while (sent < nst && sent < (R - 1) * kGroups) send();
+        }
+        int i = g;
+        for (int turn = 0; i < nst; i += kGroups, ++turn) {
+            const int sl = R * g + turn % R;
+            if (turn > 0) ok = __all_sync(FULL, mbar_wait(&empty[(i - kGroups) % SB], (i - kGroups) / SB & 1)) && ok;
+            if (ok) {
+#pragma unroll
+                for (int j = 0; j < kATileBytes / 16 / 128; ++j) st_shared_zero16(at + t * 16 + 2048 * j);
+            }
+            ok = bar_all(1 + g, 128, ok);
+            if (!ok) break;
+            if (t == 0 && sent < nst) send();
+            ok = __all_sync(FULL, mbar_wait(&efull[sl], turn / R & 1));
+            const int4 h = ok ? hdr[sl] : make_int4(0, 0, 0, 0);
+            const uint32_t *e = ring + sl * kSlot + h.x + t;
+            auto put = [&](uint32_t w) { st_shared_u16(at + (w & 0xffffu), (uint16_t)(w >> 16)); };
+            int n = h.y;
+#pragma unroll 1
+            for (; n >= 512; n -= 512, e += 512) {
+                const uint32_t w0 = e[0], w1 = e[128], w2 = e[256], w3 = e[384];
+                put(w0);
+                put(w1);
+                put(w2);
+                put(w3);
+            }
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[j] = t + 128 * j < n ? e[128 * j] : 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (t + 128 * j < n) put(w[j]);
+            for (int x = h.z + h.y + t; x < h.w; x += 128) put(__ldcs(a.t.ent + x));  // past the slot's words
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[i % SB]);
+            // the previous accumulator: complete before this stage's turn comes again
+            if (turn / kTurns > drained) drain(drained++);
+        }
+        while (ok && drained < nchunks) drain(drained++);
+        if (!ok) {
+            *failed = 1;
+            if (t == 0)  // copies still on their way land before the CTA can leave
+                for (int x = i; x < sent; x += kGroups)
+                    mbar_wait(&efull[R * g + x / kGroups % R], x / kGroups / R & 1);
+        }
+    } else if (warp == kWorkers) {
+        if (lane == 0) {
+            int issued = 0;
+            for (int i = 0; i < nst; ++i) {
+                const int s = i % SB;
+                if (i >= SB && !mbar_wait(&empty[s], (i / SB - 1) & 1)) {
+                    *failed = 1;
+                    break;
+                }
+                if (i == a.withhold && b == 0) break;  // nothing will complete full[s]
+                mbar_expect_tx(&full[s], SH::BT);
+#pragma unroll
+                for (int f = 0; f < NT / 64; ++f)
+                    tma_load_2d(bring + s * SH::BT + f * (kCols * 128), &tmB, &full[s], n0 + 64 * f, i * kCols);
+                issued = i + 1;
+            }
+            // every issued copy lands before the CTA can leave (bounded waits)
+            for (int i = issued - SB > 0 ? issued - SB : 0; i < issued; ++i) mbar_wait(&full[i % SB], (i / SB) & 1);
+        }
+    } else {
+        // The whole warp walks the loop and one elected lane issues: the descriptors then stay in
+        // uniform registers (a loop inside one lane's branch took about 80 clocks per MMA).
+        // FP32 accumulator, BF16 A (K-major) and B (MN-major: transpose bit 16), M = 128, N = NT
+        constexpr uint32_t kIdesc =
+            (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(NT >> 3) << 17) | ((128u >> 4) << 24);
+        const uint64_t ad0 = smem_desc(smem_u32(smem), 16, 1024), bd0 = smem_desc(smem_u32(bring), kCols * 128, 1024);
+        const bool one = elect_one();
+        bool ok = true;
+        for (int i = 0; i < nst; ++i) {
+            const int s = i % SB, c = i / kChunk;
+            if (i % kChunk == 0 && c >= 2) ok = __all_sync(FULL, mbar_wait(&bfree[c & 1], ((c >> 1) - 1) & 1));
+            ok = ok && __all_sync(FULL, mbar_wait(&full[s], (i / SB) & 1));
+            if (!ok) break;
+            fence_after_sync();
+            const uint64_t ad = ad0 + (uint32_t)(i % S) * (kATileBytes >> 4), bd = bd0 + (uint32_t)s * (SH::BT >> 4);
+            if (one) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    mma_bf16(taddr + (c & 1) * NT, ad + j * 2, bd + j * 128, kIdesc, (i % kChunk || j) ? 1u : 0u);
+                mma_commit(&empty[s]);
+                if (i % kChunk == kChunk - 1 || i == nst - 1) mma_commit(&cdone[c & 1]);
+            }
+            __syncwarp();
+        }
+        if (!ok && one) *failed = 1;
+    }
+    __syncwarp();
+    bool fine = true;
+    if (warp < kWorkers) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            if constexpr (P == 2) acc[0][k] += acc[1][k];
+            fine &= (__float_as_uint(acc[0][k]) & 0x7f800000u) != 0x7f800000u;
+        }
+    }
+    fence_before_sync();
+    fine = __syncthreads_and(fine);
+    fence_after_sync();
+    if (warp == 0) tmem_dealloc(taddr, 2 * NT);
+    if (tid == 0) {
+        a.marks[blockIdx.y * gridDim.x + b] = *failed || !fine;
+        if (*failed && a.err) atomicExch(a.err, 1);
+    }
+    if (*failed || !fine) return;
+    const int row = b * kRows + 32 * (warp & 3) + lane;
+    if (warp >= kWorkers || row >= a.M) return;
+    const int c0 = n0 + (warp >> 2) * W;
+    float *dst = a.C + (int64_t)row * a.ldc + c0;
+#pragma unroll
+    for (int k = 0; k < W; k += 8) {
+        if (c0 + k >= a.N) break;
+        if (a.vec == 8) {
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + k), "f"(acc[0][k]),
+                         "f"(acc[0][k + 1]), "f"(acc[0][k + 2]), "f"(acc[0][k + 3]), "f"(acc[0][k + 4]), "f"(acc[0][k + 5]),
+                         "f"(acc[0][k + 6]), "f"(acc[0][k + 7])
+                         : "memory");
+        } else if (a.vec == 4) {
+            *reinterpret_cast<float4 *>(dst + k) = make_float4(acc[0][k], acc[0][k + 1], acc[0][k + 2], acc[0][k + 3]);
+            *reinterpret_cast<float4 *>(dst + k + 4) = make_float4(acc[0][k + 4], acc[0][k + 5], acc[0][k + 6], acc[0][k + 7]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) dst[k + j] = acc[0][k + j];
+        }
+    }
+}
+
+// The marked row blocks, from the CSR arrays: a warp per row, 256 columns per pass (N a
+// multiple of 8).  Usually no block is marked and the CTAs leave at once.
+__global__ void __launch_bounds__(256) marked_rows_kernel(const SpmmProblem P, const int32_t *marks, int nb, int tiles,
+                                                          int vec_c) {
+    int marked = 0;
+    for (int y = 0; y < tiles; ++y) marked |= __ldg(marks + y * nb + blockIdx.x / (kRows / 8));
+    if (!marked) return;
+    const int lane = threadIdx.x & 31;
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row >= P.M) return;
+    const int64_t p0 = __ldg(P.rowptr + row), p1 = __ldg(P.rowptr + row + 1);
+    const int col = blockIdx.y * 256 + lane * 8;
+    float acc[1][8] = {};
+    spmm_detail::gather_range<BF16, 32, 1, 8, true>(P, p0, p1, acc, lane, col);
+    float *dst = P.C + (int64_t)row * P.ldc;
+    if (vec_c) {
+        spmm_detail::store_row<BF16, 32, 1>(dst, acc, lane, col, P.N, 1.0f);
+    } else if (col < P.N) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dst[col + k] = acc[0][k];
+    }
+}
+
+template <int NT>
+int launch_nt(const CUtensorMap &map, const Args &a, int nb, cudaStream_t s) {
+    using SH = Shape<NT>;
+    static std::once_flag once[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return fail(GBSP_ERR_UNSUPPORTED, "tc dense: device ordinal %d", dev);
+    std::call_once(once[dev], [] {
+        cudaFuncSetAttribute(spmm_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SH::SMEM);
+    });
+    spmm_kernel<NT><<<dim3((unsigned)nb, (unsigned)((a.N + NT - 1) / NT)), kThreads, SH::SMEM, s>>>(map, a);
+    count_launches(1);
+    return check_launch("tc dense spmm kernel");
+}
+
+}  // namespace
+
+bool tiles_fit(int64_t M, int64_t K) {
+    return M > 0 && K > 0 && col_tiles(K) <= kMaxTiles && row_blocks(M) * (col_tiles(K) + 1) < (1LL << 31);
+}
+
+// Time against time, in microseconds: a tile takes 0.30 / 0.38 / 0.46 at 64 / 128 / 256 features
+// whatever it holds, one CTA per SM, and a pair of launches 5 (measured on 2,048 to 24,000 rows and
+// columns); the plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 /
+// 256 features where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On
+// 16,384^2 the lines cross near 6.5% / 5% / 3% of entries.  Narrow rows are summed by more lane
+// groups in the CSR kernel, so that below 8% its error at N = 64 is the smaller one (7%: 9.4e-8
+// against 9.8e-8) and the plan keeps it.
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    if (M < 2048 || K < 2048 || N < 64 || N > 512 || (double)nnz < (N < 128 ? 0.08 : 0.03) * (double)M * (double)K)
+        return false;
+    const int sms = sm_count();
+    if (sms < 1) return false;
+    const int64_t waves = (row_blocks(M) * ((N + 255) / 256) + sms - 1) / sms;
+    const double dense = (double)(waves * col_tiles(K)) * (N <= 64 ? 0.30 : N <= 128 ? 0.38 : 0.46) + 5.0;
+    return dense < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+}
+
+int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
+               cudaStream_t s) {
+    const int nkt = (int)col_tiles(K);
+    bin_kernel<<<(unsigned)row_blocks(M), kBinThreads, sizeof(int32_t) * nkt, s>>>(rowptr, colidx, vals, (int)M, (int)K,
+                                                                                   nkt, t);
+    count_launches(1);
+    return check_launch("tc dense bin kernel");
+}
+
+int launch_spmm(const SpmmProblem &p, Tiles t, int32_t *marks, int *err, int withhold, cudaStream_t s) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return fail(GBSP_ERR_CUDA, "tc dense: cuTensorMapEncodeTiled is not available");
+    CUtensorMap map;
+    const cuuint64_t dims[2] = {(cuuint64_t)p.N, (cuuint64_t)p.K};
+    const cuuint64_t strides[1] = {(cuuint64_t)p.ldb * 2};
+    const int nt = p.N <= 64 ? 64 : p.N <= 128 ? 128 : 256;
+    const cuuint32_t box[2] = {64, kCols};
+    const cuuint32_t estr[2] = {1, 1};
+    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p.B), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return fail(GBSP_ERR_CUDA, "tc dense: tensor map encoding failed");
+    const bool c16 = aligned16(p.C) && p.ldc % 4 == 0;
+    Args a{t, marks, p.C, p.ldc, p.M, p.N, (int)col_tiles(p.K), aligned32(p.C) && p.ldc % 8 == 0 ? 8 : c16 ? 4 : 1, err,
+           withhold};
+    const int nb = (int)row_blocks(p.M);
+    int st = nt == 64 ? launch_nt<64>(map, a, nb, s) : nt == 128 ? launch_nt<128>(map, a, nb, s)
+                                                                  : launch_nt<256>(map, a, nb, s);
+    if (st) return st;
+    marked_rows_kernel<<<dim3((unsigned)nb * (kRows / 8), (unsigned)((p.N + 255) / 256)), 256, 0, s>>>(
+        p, marks, nb, (p.N + nt - 1) / nt, c16);
+    count_launches(1);
+    return check_launch("tc dense marked rows");
+}
+
+}  // namespace dense
+}  // namespace gbsp

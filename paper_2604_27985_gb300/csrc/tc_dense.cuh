@@ -1,0 +1,43 @@
+// Densified tensor-core path: A's 128 x 64 tiles are expanded into shared memory and multiplied
+// whole (tc_dense.cu).
+#pragma once
+
+#include "tc_ptx.cuh"
+
+namespace gbsp {
+namespace dense {
+
+constexpr int kRows = 128;  // rows of a block (the MMA's M)
+constexpr int kCols = 64;   // columns of a tile: 128 bytes of BF16, one swizzle atom
+
+inline int64_t row_blocks(int64_t M) { return (M + kRows - 1) / kRows; }
+inline int64_t ent_count(int64_t nnz) { return nnz + 4; }
+inline int64_t col_tiles(int64_t K) { return (K + kCols - 1) / kCols; }
+
+// A's stored entries regrouped by tile, block after block (a block's entries keep the CSR range
+// of its rows): ent[e] = BF16 value << 16 | byte offset in the swizzled tile, and
+// tptr[b * (col_tiles + 1) + t] = first entry of tile t of row block b.  bad[b] is 1 where a
+// row of the block has column indices that are not strictly increasing or not in [0, K), and
+// the block's entries are then not written.
+// ent is 16-byte aligned and has room for ent_count(nnz) words (whole 16-byte pieces are read).
+struct Tiles {
+    uint32_t *ent;
+    int32_t *tptr;
+    int32_t *bad;
+};
+
+// Whether the regrouping is possible for these sizes, and whether it is worth it.
+bool tiles_fit(int64_t M, int64_t K);
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz);
+
+int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
+               cudaStream_t s);
+// C = A B for N a multiple of 8 and 16-byte aligned B rows: every block of rows on the tensor
+// cores, then the marked ones (by t.bad when given, by a value that is not finite or by a wait
+// that ran out) again on the CUDA cores from p's CSR arrays.  marks: mark_count ints of scratch.
+// err, when given, records a wait that ran out (withhold >= 0: block 0 never loads that tile).
+inline int64_t mark_count(int64_t M, int64_t N) { return row_blocks(M) * ((N + 255) / 256); }
+int launch_spmm(const SpmmProblem &p, Tiles t, int32_t *marks, int *err, int withhold, cudaStream_t s);
+
+}  // namespace dense
+}  // namespace gbsp

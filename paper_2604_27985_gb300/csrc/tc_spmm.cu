@@ -17,11 +17,9 @@
 // 1 KB swizzled atom; rows past K are zero-filled, which also serves the padding blocks);
 // the value tile of each stage arrives by one bulk copy.  The epilogue reads TMEM and adds
 // the window's 16 rows into C.
-#include <cuda.h>
-
 #include <mutex>
 
-#include "common.cuh"
+#include "tc_dense.cuh"
 
 namespace gbsp {
 
@@ -35,134 +33,6 @@ constexpr int kATile = 2048;   // bytes of one stage of window values: 16 rows x
 // Dense blocks per pipeline stage: 8 for BF16 (64 condensed columns), 16 for E4M3 (128).
 template <bool FP8>
 constexpr int blocks_per_stage() { return FP8 ? 16 : 8; }
-constexpr uint64_t kWaitNs = 1000000000ull;  // a bounded wait gives up after one second
-
-// ---- PTX wrappers ---------------------------------------------------------------------------
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t global_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Waits for the phase with the given parity to complete; false after about a second.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_try_wait(bar, parity))
-        if (global_ns() - t0 > kWaitNs) return false;
-    return true;
-}
-
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// One box of a 3-D view of B: (128-byte feature atoms, rows, atoms) with the atoms
-// outermost, so one copy lands a dense block's 8 rows as NFA consecutive 1 KB MN-major atoms.
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-            "r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-
-// 32 TMEM lanes (one per thread of the warp) x 16 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// Shared-memory matrix descriptor (128-byte swizzle): start address, leading and stride
-// byte offsets (all >> 4), descriptor version 1, swizzle mode 2 in bits 61-63.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (2ull << 61);
-}
 
 // Instruction descriptors: FP32 accumulator, A MN-major (feature-contiguous B rows), B
 // K-major (condensed window rows), M = 128, N = 16; kind::f16 with BF16 A and B (format 1),
@@ -806,6 +676,8 @@ struct gbsp_plan {
     int withhold;  // see gbsp_plan_test_withhold
     gbsp_opts residual_opts;
     int residual_auto;  // the split AUTO chose for the residual at creation (0: not measured)
+    dense::Tiles tiles;  // BF16: every entry by 128 x 64 tile (tc_dense.cu), null where that does not pay
+    uint16_t *vals_full; // ... and A's values in CSR order
 };
 
 namespace {
@@ -838,29 +710,14 @@ void plan_free(gbsp_plan *p) {
     cudaFree(p->res_pos);
     cudaFree(p->rowptr_full);
     cudaFree(p->colidx_full);
+    cudaFree(p->tiles.ent);
+    cudaFree(p->tiles.tptr);
+    cudaFree(p->tiles.bad);
+    cudaFree(p->vals_full);
     cudaFree(p->err);
     delete p;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
 
 template <int NT, bool FP8>
 int launch_tc(const CUtensorMap &map, const TcArgs &args, int nwin, int ngroups, cudaStream_t s) {
@@ -896,6 +753,8 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     if (A->nnz > 0 && (!A->colidx || !A->vals)) return fail(GBSP_ERR_INVALID_ARG, "plan: null colidx / vals");
     // defaults measured on 16,384^2 at 90% (N = 256), uniform and clustered: the E4M3 residual
     // runs on ALU-bound CSR kernels, so sparser blocks still pay on the tensor cores
+    const bool by_default = threshold < 1 && (!residual_opts || (residual_opts->variant == GBSP_VARIANT_AUTO &&
+                                                                 !residual_opts->vecs && !residual_opts->unroll));
     if (threshold < 1) threshold = A->dtype == GBSP_E4M3 ? 10 : 14;
     const int64_t M = A->rows, K = A->cols;
     const int64_t nwin = (M + kBR - 1) / kBR, nbc = (K + kBC - 1) / kBC;
@@ -1011,6 +870,16 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
         count_launches(1);
         GBSP_TRY(check_launch("plan residual"));
     }
+    // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
+    // the plan: at a few percent of entries and more, whole tiles on the tensor cores
+    if (!fp8 && by_default && dense::tiles_fit(M, K) && dense::spmm_pays(M, K, 256, p->nnz)) {
+        GBSP_TRY(dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)));
+        GBSP_TRY(dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))));
+        GBSP_TRY(dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)));
+        GBSP_TRY(dev_alloc(&p->vals_full, (size_t)p->nnz));
+        cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
+        GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, static_cast<const uint16_t *>(A->vals), M, K, p->tiles, s));
+    }
     if (cudaStreamSynchronize(s) != cudaSuccess) GBSP_TRY(check_launch("plan sync"));
     if (p->residual_opts.variant == GBSP_VARIANT_AUTO && M > 0) {
         // the residual's automatic split is measured here, where the stream is synchronised
@@ -1102,6 +971,26 @@ GBSP_EXPORT int gbsp_plan_execute(const gbsp_plan *p, const gbsp_dense *B, gbsp_
                                           "of %d and a 16-byte aligned B",
                     amul);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    void *marks = nullptr;
+    if (p->tiles.ent && dense::spmm_pays(p->M, p->K, N, p->nnz) &&
+        scratch_alloc(&marks, sizeof(int32_t) * (size_t)dense::mark_count(p->M, N), s) == GBSP_OK) {
+        SpmmProblem q{};
+        q.M = (int32_t)p->M;
+        q.K = (int32_t)p->K;
+        q.N = (int32_t)N;
+        q.nnz = p->nnz;
+        q.rowptr = p->rowptr_full;
+        q.colidx = p->colidx_full;
+        q.vals = p->vals_full;
+        q.B = B->data;
+        q.ldb = B->ld;
+        q.C = static_cast<float *>(C->data);
+        q.ldc = C->ld;
+        q.dtype = GBSP_BF16;
+        const int st = dense::launch_spmm(q, p->tiles, static_cast<int32_t *>(marks), p->err, p->withhold, s);
+        scratch_free(marks, s);
+        return st ? st : ok();
+    }
     // residual entries (and the overwrite of C) through the CSR kernels
     gbsp_csr R{p->M, p->K, p->res_nnz, p->res_rowptr, p->res_colidx, p->res_vals, p->res_scale, p->dtype};
     gbsp_opts ro = p->residual_opts;

@@ -1,0 +1,136 @@
+"""GPU parity of the densified tensor-core SpMM (128 x 64 tiles of A expanded in shared memory).
+
+Taken by a default plan of a BF16 matrix with at least 2,048 rows and columns and enough entries.
+Integer inputs (exact in BF16, partial sums below 2^24) match the oracle bit for bit; random
+ones are held to the FP32 tolerance against the oracle on the BF16-rounded operands.
+"""
+import numpy as np
+import pytest
+
+import gen
+import oracle
+from _util import assert_within, dev
+
+pytestmark = pytest.mark.gpu
+TOL32 = 1e-5
+
+
+@pytest.fixture(scope="module")
+def gb():
+    import paper_2604_27985_gb300 as g
+
+    return g
+
+
+def bf16(x):
+    import torch
+
+    return dev(oracle.bf16_round(x).view(np.int16)).view(torch.bfloat16)
+
+
+def matrix(M, K, seed, lo=0.8, hi=1.0):
+    """Rows of lo * K to hi * K entries, some empty, one full."""
+    lengths = np.random.default_rng(seed).integers(int(lo * K), int(hi * K) + 1, M)
+    lengths[::97] = 0
+    lengths[5] = K
+    return gen.csr_from_lengths(lengths, K, seed=seed)
+
+
+# Nearly full rows, so that small matrices take the path (and tiles overflow their entry slots).
+# Tile edges: M around a multiple of 128, K around one of 64 and of 256 (an accumulator), every
+# feature tile (64, 128, 256, two of 256) full and cut
+SHAPES = [(2048, 2048, 64), (2049, 2111, 72), (2175, 2049, 128), (2176, 2304, 136), (2500, 2305, 256),
+          (3001, 2624, 264), (2100, 4099, 512)]
+
+
+@pytest.mark.parametrize("M,K,N", SHAPES)
+def test_dense_integers_bit_exact(gb, M, K, N):
+    A = matrix(M, K, 700 + N)
+    vals, B = gen.vals_int(A.nnz, 701), gen.dense_int(K, N, 702)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(vals), K)
+    before = gb.launch_count()
+    C = plan.execute(bf16(B))
+    assert gb.launch_count() - before == 2  # the tile kernel and the marked rows
+    plan.check()
+    want, _ = oracle.spmm(A.rowptr, A.colidx, vals, B)
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+
+
+def test_dense_sparse_tiles(gb):
+    """12% of entries, all in the even 64-column tiles of the first 4,096 columns and in a few
+    others: tiles below a slot's size, tiles with no entry, rows with none."""
+    rng = np.random.default_rng(705)
+    M, K = 6000, 6000
+    cand = np.concatenate([np.arange(t, t + 64) for t in range(0, 4096, 128)] + [np.arange(5900, 6000)])
+    rows, cols = [], []
+    for r in range(M):
+        c = cand[rng.random(cand.size) < 0.34] if r % 50 else cand[:0]
+        rows.append(np.full(c.size, r))
+        cols.append(c)
+    rows, cols = np.concatenate(rows), np.concatenate(cols)
+    vals, B = gen.vals_int(rows.size, 706), gen.dense_int(K, 256, 707)
+    A = gen.csr_from_triplets(M, K, rows, cols, vals)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(vals), K)
+    before = gb.launch_count()
+    C = plan.execute(bf16(B))
+    assert gb.launch_count() - before == 2
+    plan.check()
+    want, _ = oracle.spmm(A.rowptr, A.colidx, vals, B)
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+
+
+def test_dense_random_padded_and_unaligned(gb):
+    import torch
+
+    A = matrix(2200, 2500, 710, 0.4, 0.8)
+    B = gen.dense_normal(2500, 200, 711)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(A.vals), 2500)
+    ref, sc = oracle.spmm(A.rowptr, A.colidx, oracle.bf16_decode(oracle.bf16_round(A.vals)),
+                          oracle.bf16_decode(oracle.bf16_round(B)))
+    wide = torch.zeros((2500, 232), dtype=torch.bfloat16, device="cuda")
+    wide[:, :200] = bf16(B)
+    for ld in (200, 204, 207):  # 32-byte, 16-byte and 4-byte aligned rows of C
+        full = torch.full((2200, ld), 7.0, device="cuda")
+        C = plan.execute(wide[:, :200], out=full[:, :200])
+        assert_within(C.cpu().numpy(), ref, sc, TOL32, f"ld {ld}")
+        assert bool((full[:, 200:] == 7.0).all())
+    plan.check()
+
+
+def test_dense_infinities_and_nan_stay_in_their_rows(gb):
+    """An infinity or NaN in a B row reaches only the rows of C that store an entry there."""
+    A = matrix(2304, 2112, 720)
+    vals, B = gen.vals_int(A.nnz, 721), gen.dense_int(2112, 64, 722)
+    B[100, 3], B[2000, 60] = np.inf, np.nan
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(vals), 2112)
+    C = plan.execute(bf16(B)).cpu().numpy()
+    plan.check()
+    Z = B.copy()
+    Z[100, 3] = Z[2000, 60] = 0
+    want, _ = oracle.spmm(A.rowptr, A.colidx, vals, Z)
+    rows = np.repeat(np.arange(A.M), np.diff(A.rowptr))
+    hit_inf, hit_nan = np.zeros(A.M, bool), np.zeros(A.M, bool)
+    hit_inf[rows[A.colidx == 100]] = True
+    hit_nan[rows[A.colidx == 2000]] = True
+    assert hit_inf.any() and hit_nan.any() and not hit_inf.all()
+    assert np.array_equal(~np.isfinite(C[:, 3]), hit_inf) and np.array_equal(np.isnan(C[:, 60]), hit_nan)
+    C[hit_inf, 3], C[hit_nan, 60] = want[hit_inf, 3], want[hit_nan, 60]
+    assert np.array_equal(C.astype(np.float64), want)
+
+
+def test_dense_bounded_wait_reports_timeout(gb):
+    """A tile whose B rows never arrive: the waits give up, the plan reports the timeout, and
+    the block's rows are computed again on the CUDA cores."""
+    A = matrix(2048, 2048, 730)
+    vals, B = gen.vals_int(A.nnz, 731), gen.dense_int(2048, 64, 732)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(vals), 2048)
+    want, _ = oracle.spmm(A.rowptr, A.colidx, vals, B)
+    plan.test_withhold(5)
+    C = plan.execute(bf16(B))
+    with pytest.raises(gb.GbspError, match="TIMEOUT"):
+        plan.check()
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+    plan.test_withhold(-1)
+    C = plan.execute(bf16(B))
+    plan.check()
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
