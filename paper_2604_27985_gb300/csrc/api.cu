@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tc_dense.cuh"
 
 namespace gbsp {
 
@@ -146,6 +147,46 @@ bool vec_ok(const gbsp_dense *D) {
     return aligned16(D->data) && D->ld % V == 0 && D->cols % V == 0;
 }
 
+SpmmProblem spmm_problem(const gbsp_csr &A, const gbsp_dense &B, const gbsp_dense &C) {
+    SpmmProblem p{};
+    p.M = (int32_t)A.rows;
+    p.K = (int32_t)A.cols;
+    p.N = (int32_t)B.cols;
+    p.nnz = A.nnz;
+    p.rowptr = A.rowptr;
+    p.colidx = A.colidx;
+    p.vals = A.vals;
+    p.a_scale = A.row_scale;
+    p.B = B.data;
+    p.ldb = B.ld;
+    p.b_scale = B.row_scale;
+    p.C = static_cast<float *>(C.data);
+    p.ldc = C.ld;
+    p.dtype = A.dtype;
+    return p;
+}
+
+// The whole-tile tensor-core SpMM of a call without a plan: the entries are regrouped by tile
+// into scratch first.  done stays false, and nothing is queued, where the scratch cannot be had
+// or the stream is being captured (a graph would hold the scratch of every replay).
+int spmm_dense(const gbsp_csr &A, const gbsp_dense &B, const gbsp_dense &C, cudaStream_t s, bool *done) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return check_launch("spmm: capture status");
+    if (cap != cudaStreamCaptureStatusNone) return GBSP_OK;
+    const int64_t nent = (dense::ent_count(A.nnz) + 3) & ~3LL, nb = dense::row_blocks(A.rows);
+    const int64_t nptr = nb * (dense::col_tiles(A.cols) + 1);
+    void *w = nullptr;
+    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(nent + nptr + nb + dense::mark_count(A.rows, B.cols)), s))
+        return GBSP_OK;
+    int32_t *i32 = static_cast<int32_t *>(w);
+    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + nent, i32 + nent + nptr};
+    int st = dense::launch_bin(A.rowptr, A.colidx, static_cast<const uint16_t *>(A.vals), A.rows, A.cols, t, s);
+    if (!st) st = dense::launch_spmm(spmm_problem(A, B, C), t, i32 + nent + nptr + nb, nullptr, -1, s);
+    scratch_free(w, s);
+    *done = true;
+    return st;
+}
+
 }  // namespace
 }  // namespace gbsp
 
@@ -182,6 +223,13 @@ GBSP_EXPORT int spmm_csr_ex(const gbsp_csr *A, const gbsp_dense *B, gbsp_dense *
         variant = GBSP_VARIANT_SCALAR;
         const int64_t rb = B->cols * elem_bytes(B->dtype);
         if (vec && (st = auto_choice(*A, kOpSpmm, B->rows * rb, rb, s, &variant, nullptr))) return st;
+        if (variant == GBSP_VARIANT_ROWSPLIT && !o.vecs && !o.unroll && A->dtype == GBSP_BF16 && A->nnz > 0 &&
+            dense::tiles_fit(A->rows, A->cols) &&
+            dense::spmm_pays_unplanned(A->rows, A->cols, B->cols, A->nnz)) {
+            bool done = false;
+            if ((st = spmm_dense(*A, *B, *C, s, &done))) return st;
+            if (done) return ok();
+        }
     }
     if (variant != GBSP_VARIANT_SCALAR && !vec)
         return fail(GBSP_ERR_ALIGN, "spmm: vectorised variant needs 16-byte aligned B and C, and N and ld "
@@ -193,21 +241,7 @@ GBSP_EXPORT int spmm_csr_ex(const gbsp_csr *A, const gbsp_dense *B, gbsp_dense *
                                           "plan entry points");
     if (variant < GBSP_VARIANT_ROWSPLIT || variant > GBSP_VARIANT_ROWGROUP)
         return fail(GBSP_ERR_INVALID_ARG, "spmm: unknown variant %d", variant);
-    SpmmProblem p{};
-    p.M = (int32_t)A->rows;
-    p.K = (int32_t)A->cols;
-    p.N = (int32_t)B->cols;
-    p.nnz = A->nnz;
-    p.rowptr = A->rowptr;
-    p.colidx = A->colidx;
-    p.vals = A->vals;
-    p.a_scale = A->row_scale;
-    p.B = B->data;
-    p.ldb = B->ld;
-    p.b_scale = B->row_scale;
-    p.C = static_cast<float *>(C->data);
-    p.ldc = C->ld;
-    p.dtype = A->dtype;
+    const SpmmProblem p = spmm_problem(*A, *B, *C);
     if ((st = launch_spmm(p, variant, o.vecs, o.unroll, o.ctas_per_sm, s))) return st;
     return ok();
 }

@@ -47,41 +47,73 @@ using namespace gbsp::tc;
 
 // ---- regrouping -----------------------------------------------------------------------------
 
+constexpr int kColBits = 6;  // log2(kCols)
+static_assert(1 << kColBits == kCols, "tiles of 64 columns");
 constexpr int kBinThreads = 1024;
-constexpr int kMaxTiles = 8 * 1024;   // one shared-memory counter per tile of a row block
+constexpr int kMaxTiles = 8 * 1024;  // one shared-memory counter per tile of a row block
 
-// Runs f(column, run length, first lane of the run, lane of this entry) over 32 entries of a row
-// at a time; a run is a maximal stretch of entries in one tile (a run cut by a chunk's end is
-// two runs).  Returns false when the columns are not strictly increasing in [0, K).
-template <class F>
-__device__ __forceinline__ bool for_runs(const int32_t *colidx, int64_t p0, int64_t p1, int K, int lane, F f) {
-    bool good = true;
-    for (int64_t base = p0; base < p1; base += 32) {
-        const int64_t p = base + lane;
-        const bool in = p < p1;
-        const int c = in ? __ldg(colidx + p) : 0x7fffffff;
-        int prev = __shfl_up_sync(FULL, c, 1);
-        if (lane == 0) prev = base > p0 ? __ldg(colidx + base - 1) : -1;
-        if (in && (c <= prev || c < 0 || c >= K)) good = false;
-        const unsigned heads =
-            __ballot_sync(FULL, in && (lane == 0 || (c / kCols) != (prev / kCols)));
-        const int cnt = p1 - base < 32 ? (int)(p1 - base) : 32;
-        const unsigned upto = heads & (FULL >> (31 - lane));
-        const int first = upto ? 31 - __clz(upto) : 0;
-        const unsigned after = lane == 31 ? 0u : heads & (FULL << (lane + 1));
-        const int end = after ? __ffs(after) - 1 : cnt;
-        f(p, in && c >= 0 && c < K, c, first, end - first);
+// Entries [p0, p1) of a row, U chunks of 32 at a time with the next U chunks' loads in flight:
+// f(columns, values, first entry of the first chunk, whether every lane holds an entry).  Lanes past
+// p1 hold column kNone.
+constexpr int kNone = 0x7fffffff;
+struct true_t { static constexpr bool value = true; };
+struct false_t { static constexpr bool value = false; };
+template <int U, bool VALS, class F>
+__device__ __forceinline__ void for_chunks(const int32_t *colidx, const uint16_t *vals, int p0, int p1, int lane,
+                                           F f) {
+    int nc[U];
+    uint16_t nv[U];
+    const int32_t *cp = colidx + p0 + lane;
+    const uint16_t *vp = vals + p0 + lane;
+    auto load = [&](int left) {  // (left entries of the row from the next block's first one on)
+        if (left >= 32 * U) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                nc[u] = __ldg(cp + 32 * u);
+                if (VALS) nv[u] = __ldg(vp + 32 * u);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool in = 32 * u + lane < left;
+                nc[u] = in ? __ldg(cp + 32 * u) : kNone;
+                if (VALS) nv[u] = in ? __ldg(vp + 32 * u) : 0;
+            }
+        }
+        cp += 32 * U;
+        vp += 32 * U;
+    };
+    load(p1 - p0);
+    for (int base = p0; base < p1; base += 32 * U) {
+        int c[U];
+        uint16_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            c[u] = nc[u];
+            v[u] = VALS ? nv[u] : 0;
+        }
+        if (base + 32 * U < p1) load(p1 - base - 32 * U);
+        if (base + 32 * U <= p1)
+            f(c, v, base, true_t{});
+        else
+            f(c, v, base, false_t{});
     }
-    return __all_sync(FULL, good);
 }
 
-// One CTA per block of 128 rows: counts the entries per tile, turns the counts into offsets and
-// writes each entry's packed word at the tile's cursor (the order inside a tile is free: every
-// entry has its own place in the tile).
+// One CTA per block of 128 rows, a warp per row: counts the entries per tile, turns the counts into
+// offsets and writes each entry's packed word at its tile's cursor (the order inside a tile is
+// free: every entry has its own place there).  The two passes read the column indices from HBM
+// and again mostly from L2.  Columns ascend, so a tile's count is the sum over rows of where the
+// row leaves the tile minus where it enters it; a chunk's run of entries in one tile is placed by
+// its first lane's reservation.
+// 16,384^2 at 90% (26.8M entries): 107 us, bound by instruction issue (89 per 32 entries); 168 with
+// the runs also counted and one chunk in flight.  Three launches over a table of every row's
+// entry into every tile, with the whole GPU but no atomics, took 53 + 16 + 69.
 __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restrict__ rowptr,
                                                           const int32_t *__restrict__ colidx,
                                                           const uint16_t *__restrict__ vals, int M, int K, int nkt,
                                                           Tiles t) {
+    constexpr int U = 4;
     extern __shared__ int32_t cnt[];  // nkt counters, then cursors
     __shared__ int32_t warp_sum[32];
     __shared__ int32_t carry;
@@ -91,11 +123,30 @@ __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restr
     if (tid == 0) carry = 0;
     __syncthreads();
     bool good = true;
-    for (int r = r0 + warp; r < r1; r += kBinThreads / 32)
-        good &= for_runs(colidx, __ldg(rowptr + r), __ldg(rowptr + r + 1), K, lane,
-                         [&](int64_t, bool in, int c, int first, int len) {
-                             if (in && first == lane) atomicAdd(&cnt[c / kCols], len);
-                         });
+    for (int r = r0 + warp; r < r1; r += kBinThreads / 32) {
+        const int p0 = __ldg(rowptr + r), p1 = __ldg(rowptr + r + 1);
+        int last = -1;  // the column before the chunk's first
+        for_chunks<U, false>(colidx, nullptr, p0, p1, lane, [&](const int (&c)[U], const uint16_t (&)[U], int base, auto all) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                int prev = __shfl_up_sync(FULL, c[u], 1);
+                if (lane == 0) prev = last;
+                last = __shfl_sync(FULL, c[u], 31);
+                if (!all.value && c[u] == kNone) continue;
+                const bool fits = c[u] > prev && c[u] < K;
+                good &= fits;
+                const int p = base + 32 * u + lane, t1 = c[u] >> kColBits, t0 = prev >> kColBits;
+                if (fits && t1 != t0) {
+                    atomicSub(&cnt[t1], p);
+                    if (t0 >= 0 && t0 < nkt) atomicAdd(&cnt[t0], p);
+                }
+            }
+        });
+        if (lane == 0 && p1 > p0) {
+            const int c = __ldg(colidx + p1 - 1);
+            if (c >= 0 && c < K) atomicAdd(&cnt[c >> kColBits], p1);
+        }
+    }
     const bool bad = !__syncthreads_and(good);
     const int32_t start = __ldg(rowptr + r0);
     int32_t *tp = t.tptr + (int64_t)b * (nkt + 1);
@@ -125,18 +176,30 @@ __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restr
         t.bad[b] = bad ? 1 : 0;
     }
     if (bad) return;
-    for (int r = r0 + warp; r < r1; r += kBinThreads / 32)
-        for_runs(colidx, __ldg(rowptr + r), __ldg(rowptr + r + 1), K, lane,
-                 [&](int64_t p, bool in, int c, int first, int len) {
-                     int at = 0;
-                     if (in && first == lane) at = atomicAdd(&cnt[c / kCols], len);
-                     at = __shfl_sync(FULL, at, first) + lane - first;
-                     if (in) {
-                         const int rr = r - r0, cc = c % kCols;
-                         const uint32_t off = rr * 128 + (((cc >> 3) ^ (rr & 7)) << 4) + (cc & 7) * 2;
-                         t.ent[at] = ((uint32_t)__ldg(vals + p) << 16) | off;
-                     }
-                 });
+    const unsigned upto = FULL >> (31 - lane), beyond = ~upto;
+    for (int r = r0 + warp; r < r1; r += kBinThreads / 32) {
+        const uint32_t row_off = (r - r0) * 128, flip = ((r - r0) & 7) << 4;
+        for_chunks<U, true>(colidx, vals, __ldg(rowptr + r), __ldg(rowptr + r + 1), lane,
+                            [&](const int (&c)[U], const uint16_t (&v)[U], int, auto all) {
+            int first[U], at[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int t1 = c[u] >> kColBits, t0 = __shfl_up_sync(FULL, t1, 1);
+                const unsigned heads = __ballot_sync(FULL, t1 != t0) | 1u;
+                first[u] = 31 - __clz(heads & upto);
+                if (first[u] == lane && (all.value || c[u] != kNone)) {  // (lanes without an entry are a run too)
+                    const unsigned after = heads & beyond;
+                    at[u] = atomicAdd(&cnt[t1], (after ? __ffs(after) - 1 : 32) - lane) - lane;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int to = __shfl_sync(FULL, at[u], first[u]) + lane;
+                const uint32_t off = row_off + (((uint32_t)c[u] << 1 & 0x70u) ^ flip) + ((uint32_t)c[u] << 1 & 0xeu);
+                if (all.value || c[u] != kNone) t.ent[to] = ((uint32_t)v[u] << 16) | off;
+            }
+        });
+    }
 }
 
 // ---- product --------------------------------------------------------------------------------
@@ -511,21 +574,44 @@ bool tiles_fit(int64_t M, int64_t K) {
     return M > 0 && K > 0 && col_tiles(K) <= kMaxTiles && row_blocks(M) * (col_tiles(K) + 1) < (1LL << 31);
 }
 
+
 // Time against time, in microseconds: a tile takes 0.30 / 0.38 / 0.46 at 64 / 128 / 256 features
 // whatever it holds, one CTA per SM, and a pair of launches 5 (measured on 2,048 to 24,000 rows and
-// columns); the plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 /
-// 256 features where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On
-// 16,384^2 the lines cross near 6.5% / 5% / 3% of entries.  Narrow rows are summed by more lane
-// groups in the CSR kernel, so that below 8% its error at N = 64 is the smaller one (7%: 9.4e-8
-// against 9.8e-8) and the plan keeps it.
+// columns).
+static double product_us(int64_t M, int64_t K, int64_t N, int64_t *waves) {
+    const int sms = sm_count() > 0 ? sm_count() : 1;
+    *waves = (row_blocks(M) * ((N + 255) / 256) + sms - 1) / sms;
+    return (double)(*waves * col_tiles(K)) * (N <= 64 ? 0.30 : N <= 128 ? 0.38 : 0.46) + 5.0;
+}
+
+// The CSR kernels split a row among 8, 4 or 2 lane groups at 64, 128 or 256 features, so short rows
+// are summed there with the smaller error: the two are level near 600 entries a row at N = 128
+// (7% of 8,192 columns: 8.2e-8 both) and near 300 at N = 256 (7% of 4,096: 7.7e-8 both).
+static bool sums_as_well(int64_t M, int64_t N, int64_t nnz) {
+    return N >= 128 && nnz >= (N < 192 ? 600 : 300) * M;
+}
+
+// The plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 / 256 features
+// where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On 16,384^2 the
+// lines cross near 6.5% / 5% / 3% of entries.  From 8% on the blocks are summed over all columns
+// on the tensor cores (error 1e-7 and more at any width), below that mostly by the CSR kernels.
 bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz) {
-    if (M < 2048 || K < 2048 || N < 64 || N > 512 || (double)nnz < (N < 128 ? 0.08 : 0.03) * (double)M * (double)K)
-        return false;
-    const int sms = sm_count();
-    if (sms < 1) return false;
-    const int64_t waves = (row_blocks(M) * ((N + 255) / 256) + sms - 1) / sms;
-    const double dense = (double)(waves * col_tiles(K)) * (N <= 64 ? 0.30 : N <= 128 ? 0.38 : 0.46) + 5.0;
-    return dense < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+    const double density = (double)nnz / ((double)M * (double)K);
+    if (M < 2048 || K < 2048 || N < 64 || N > 512 || density < 0.03) return false;
+    if (density < 0.08 && !sums_as_well(M, N, nnz)) return false;
+    int64_t waves;
+    return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+}
+
+// For rows of even length (the split AUTO would take is the row split).  The regrouping takes 0.5 ns
+// per entry of a block of rows, the row split 13 / 24 ps per entry at 128 / 256 features: on
+// 16,384^2 the lines cross near 4.5% / 2.5% of entries, on 8,192^2 near 11% / 5%.
+bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    if (M < 2048 || K < 2048 || N > 512 || !sums_as_well(M, N, nnz)) return false;
+    int64_t waves;
+    const double product = product_us(M, K, N, &waves);
+    const double bins = (double)waves * 0.5e-3 * (double)nnz / (double)row_blocks(M);
+    return product + bins < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
 }
 
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
@@ -534,7 +620,7 @@ int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *val
     bin_kernel<<<(unsigned)row_blocks(M), kBinThreads, sizeof(int32_t) * nkt, s>>>(rowptr, colidx, vals, (int)M, (int)K,
                                                                                    nkt, t);
     count_launches(1);
-    return check_launch("tc dense bin kernel");
+    return check_launch("tc dense regrouping");
 }
 
 int launch_spmm(const SpmmProblem &p, Tiles t, int32_t *marks, int *err, int withhold, cudaStream_t s) {

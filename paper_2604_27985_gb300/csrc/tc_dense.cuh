@@ -29,6 +29,8 @@ struct Tiles {
 // Whether the regrouping is possible for these sizes, and whether it is worth it.
 bool tiles_fit(int64_t M, int64_t K);
 bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz);
+// ... also where the regrouping is part of every call, against the CSR kernels.
+bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz);
 
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
                cudaStream_t s);

@@ -873,12 +873,20 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
     if (!fp8 && by_default && dense::tiles_fit(M, K) && dense::spmm_pays(M, K, 256, p->nnz)) {
-        GBSP_TRY(dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)));
-        GBSP_TRY(dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))));
-        GBSP_TRY(dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)));
-        GBSP_TRY(dev_alloc(&p->vals_full, (size_t)p->nnz));
-        cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
-        GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, static_cast<const uint16_t *>(A->vals), M, K, p->tiles, s));
+        if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
+            dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
+            dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)) == GBSP_OK &&
+            dev_alloc(&p->vals_full, (size_t)p->nnz) == GBSP_OK) {
+            cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
+            GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, static_cast<const uint16_t *>(A->vals), M, K, p->tiles, s));
+        } else {  // no room: the plan works without
+            cudaFree(p->tiles.ent);
+            cudaFree(p->tiles.tptr);
+            cudaFree(p->tiles.bad);
+            cudaFree(p->vals_full);
+            p->tiles = dense::Tiles{};
+            p->vals_full = nullptr;
+        }
     }
     if (cudaStreamSynchronize(s) != cudaSuccess) GBSP_TRY(check_launch("plan sync"));
     if (p->residual_opts.variant == GBSP_VARIANT_AUTO && M > 0) {

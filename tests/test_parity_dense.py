@@ -134,3 +134,50 @@ def test_dense_bounded_wait_reports_timeout(gb):
     C = plan.execute(bf16(B))
     plan.check()
     assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+
+
+def launches(gb, f):
+    before = gb.launch_count()
+    out = f()
+    return out, gb.launch_count() - before
+
+
+@pytest.mark.parametrize("M,K,N", [(12001, 2049, 128), (12100, 2111, 136), (12032, 2304, 264)])
+def test_dense_without_a_plan(gb, M, K, N):
+    """AUTO on a BF16 matrix regroups per call: the row statistics, one launch for that, and
+    the two of a plan."""
+    A = matrix(M, K, 740 + N, 0.25, 0.4)
+    vals, B = gen.vals_int(A.nnz, 741), gen.dense_int(K, N, 742)
+    rp, ci, v, b = dev(A.rowptr), dev(A.colidx), bf16(vals), bf16(B)
+    C, n = launches(gb, lambda: gb.spmm(rp, ci, v, b))
+    assert n == 4
+    want, _ = oracle.spmm(A.rowptr, A.colidx, vals, B)
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+
+
+def test_dense_without_a_plan_any_column_order(gb):
+    """Rows with repeated or unordered columns (sums of repeats, any order) go to the CUDA cores
+    with their block of 128 rows; under capture, and with a chosen variant, nothing is regrouped."""
+    import torch
+
+    A = matrix(12032, 2304, 750, 0.25, 0.4)
+    ci = A.colidx.copy()
+    for r in (1, 700, 701):  # blocks 0 and 5
+        ci[A.rowptr[r]:A.rowptr[r + 1]] = ci[A.rowptr[r]:A.rowptr[r + 1]][::-1]
+    ci[A.rowptr[12031]] = ci[A.rowptr[12031] + 1]  # a repeat, in the last block
+    vals, B = gen.vals_int(A.nnz, 751), gen.dense_int(2304, 128, 752)
+    want, _ = oracle.spmm(A.rowptr, ci, vals, B)
+    rp, c, v, b = dev(A.rowptr), dev(ci), bf16(vals), bf16(B)
+    C, n = launches(gb, lambda: gb.spmm(rp, c, v, b))
+    assert n == 4 and np.array_equal(C.cpu().numpy().astype(np.float64), want)
+    C, n = launches(gb, lambda: gb.spmm(rp, c, v, b, variant="rowsplit"))
+    assert n == 1 and np.array_equal(C.cpu().numpy().astype(np.float64), want)
+    out = torch.zeros((12032, 128), device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    gb.auto_forget()  # (a pattern unknown under capture takes the row split)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        _, n = launches(gb, lambda: gb.spmm(rp, c, v, b, out=out))
+    assert n == 1
+    graph.replay()
+    assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
