@@ -166,6 +166,26 @@ SpmmProblem spmm_problem(const gbsp_csr &A, const gbsp_dense &B, const gbsp_dens
     return p;
 }
 
+SddmmProblem sddmm_problem(const gbsp_csr &S, const gbsp_dense &X, const gbsp_dense &Y, float *out) {
+    SddmmProblem p{};
+    p.M = (int32_t)S.rows;
+    p.N = (int32_t)S.cols;
+    p.Kd = (int32_t)X.cols;
+    p.nnz = S.nnz;
+    p.rowptr = S.rowptr;
+    p.colidx = S.colidx;
+    p.svals = static_cast<const float *>(S.vals);
+    p.X = X.data;
+    p.ldx = X.ld;
+    p.x_scale = X.row_scale;
+    p.Y = Y.data;
+    p.ldy = Y.ld;
+    p.y_scale = Y.row_scale;
+    p.out = out;
+    p.dtype = X.dtype;
+    return p;
+}
+
 // The whole-tile tensor-core SpMM of a call without a plan: the entries are regrouped by tile
 // into scratch first.  done stays false, and nothing is queued, where the scratch cannot be had
 // or the stream is being captured (a graph would hold the scratch of every replay).
@@ -179,9 +199,27 @@ int spmm_dense(const gbsp_csr &A, const gbsp_dense &B, const gbsp_dense &C, cuda
     if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(nent + nptr + nb + dense::mark_count(A.rows, B.cols)), s))
         return GBSP_OK;
     int32_t *i32 = static_cast<int32_t *>(w);
-    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + nent, i32 + nent + nptr};
+    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + nent, i32 + nent + nptr, nullptr};
     int st = dense::launch_bin(A.rowptr, A.colidx, static_cast<const uint16_t *>(A.vals), A.rows, A.cols, t, s);
     if (!st) st = dense::launch_spmm(spmm_problem(A, B, C), t, i32 + nent + nptr + nb, nullptr, -1, s);
+    scratch_free(w, s);
+    *done = true;
+    return st;
+}
+
+// ... and the SDDMM (E4M3 X and Y).
+int sddmm_dense(const gbsp_csr &S, const gbsp_dense &X, const gbsp_dense &Y, float *out, cudaStream_t s, bool *done) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return check_launch("sddmm: capture status");
+    if (cap != cudaStreamCaptureStatusNone) return GBSP_OK;
+    const int64_t nent = (dense::ent_count(S.nnz) + 3) & ~3LL, nb = dense::row_blocks(S.rows);
+    const int64_t nptr = nb * (dense::col_tiles(S.cols) + 1);
+    void *w = nullptr;
+    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(2 * nent + nptr + nb), s)) return GBSP_OK;
+    int32_t *i32 = static_cast<int32_t *>(w);
+    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + 2 * nent, i32 + 2 * nent + nptr, i32 + nent};
+    int st = dense::launch_bin(S.rowptr, S.colidx, nullptr, S.rows, S.cols, t, s);
+    if (!st) st = dense::launch_sddmm(sddmm_problem(S, X, Y, out), t, nullptr, -1, s);
     scratch_free(w, s);
     *done = true;
     return st;
@@ -275,6 +313,12 @@ GBSP_EXPORT int sddmm_csr_ex(const gbsp_csr *S, const gbsp_dense *X, const gbsp_
         variant = GBSP_VARIANT_SCALAR;
         const int64_t rb = Y->cols * elem_bytes(Y->dtype);
         if (vec && (st = auto_choice(*S, kOpSddmm, Y->rows * rb, rb, s, &variant, nullptr))) return st;
+        if (variant == GBSP_VARIANT_ROWSPLIT && !o.vecs && X->dtype == GBSP_E4M3 && S->nnz > 0 &&
+            dense::tiles_fit(S->rows, S->cols) && dense::sddmm_pays_unplanned(S->rows, S->cols, X->cols, S->nnz)) {
+            bool done = false;
+            if ((st = sddmm_dense(*S, *X, *Y, out, s, &done))) return st;
+            if (done) return ok();
+        }
     }
     if (variant != GBSP_VARIANT_SCALAR && !vec)
         return fail(GBSP_ERR_ALIGN, "sddmm: vectorised variant needs 16-byte aligned X and Y, Kd and ld "
@@ -283,22 +327,7 @@ GBSP_EXPORT int sddmm_csr_ex(const gbsp_csr *S, const gbsp_dense *X, const gbsp_
         return fail(GBSP_ERR_UNSUPPORTED, "sddmm: the row groups and the SpMM plans are SpMM variants");
     if (variant < GBSP_VARIANT_ROWSPLIT || variant > GBSP_VARIANT_ENTRY)
         return fail(GBSP_ERR_INVALID_ARG, "sddmm: unknown variant %d", variant);
-    SddmmProblem p{};
-    p.M = (int32_t)S->rows;
-    p.N = (int32_t)S->cols;
-    p.Kd = (int32_t)X->cols;
-    p.nnz = S->nnz;
-    p.rowptr = S->rowptr;
-    p.colidx = S->colidx;
-    p.svals = static_cast<const float *>(S->vals);
-    p.X = X->data;
-    p.ldx = X->ld;
-    p.x_scale = X->row_scale;
-    p.Y = Y->data;
-    p.ldy = Y->ld;
-    p.y_scale = Y->row_scale;
-    p.out = out;
-    p.dtype = X->dtype;
+    const SddmmProblem p = sddmm_problem(*S, *X, *Y, out);
     if ((st = launch_sddmm(p, variant, o.vecs, s))) return st;
     return ok();
 }

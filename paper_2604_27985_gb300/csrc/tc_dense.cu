@@ -109,6 +109,7 @@ __device__ __forceinline__ void for_chunks(const int32_t *colidx, const uint16_t
 // 16,384^2 at 90% (26.8M entries): 107 us, bound by instruction issue (89 per 32 entries); 168 with
 // the runs also counted and one chunk in flight.  Three launches over a table of every row's
 // entry into every tile, with the whole GPU but no atomics, took 53 + 16 + 69.
+template <bool VALS, bool POS>
 __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restrict__ rowptr,
                                                           const int32_t *__restrict__ colidx,
                                                           const uint16_t *__restrict__ vals, int M, int K, int nkt,
@@ -179,8 +180,8 @@ __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restr
     const unsigned upto = FULL >> (31 - lane), beyond = ~upto;
     for (int r = r0 + warp; r < r1; r += kBinThreads / 32) {
         const uint32_t row_off = (r - r0) * 128, flip = ((r - r0) & 7) << 4;
-        for_chunks<U, true>(colidx, vals, __ldg(rowptr + r), __ldg(rowptr + r + 1), lane,
-                            [&](const int (&c)[U], const uint16_t (&v)[U], int, auto all) {
+        for_chunks<U, VALS>(colidx, vals, __ldg(rowptr + r), __ldg(rowptr + r + 1), lane,
+                            [&](const int (&c)[U], const uint16_t (&v)[U], int base, auto all) {
             int first[U], at[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -196,7 +197,10 @@ __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restr
             for (int u = 0; u < U; ++u) {
                 const int to = __shfl_sync(FULL, at[u], first[u]) + lane;
                 const uint32_t off = row_off + (((uint32_t)c[u] << 1 & 0x70u) ^ flip) + ((uint32_t)c[u] << 1 & 0xeu);
-                if (all.value || c[u] != kNone) t.ent[to] = ((uint32_t)v[u] << 16) | off;
+                if (all.value || c[u] != kNone) {
+                    t.ent[to] = ((uint32_t)v[u] << 16) | off;
+                    if (POS) t.pos[to] = base + 32 * u + lane;
+                }
             }
         });
     }
@@ -232,37 +236,6 @@ struct Args {
     int *err;
     int withhold;
 };
-
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// True in one lane of a converged warp.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "elect.sync _|p, 0xffffffff;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(p));
-    return p != 0;
-}
-
-// Barrier of n threads that returns the conjunction of their votes.
-__device__ __forceinline__ bool bar_all(int id, int n, bool vote) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %3, 0;\n\t"
-        "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(id), "r"(n), "r"((uint32_t)vote)
-        : "memory");
-    return r != 0;
-}
-
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 
 __device__ __forceinline__ void st_shared_u16(uint32_t addr, uint16_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
@@ -617,8 +590,9 @@ bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
                cudaStream_t s) {
     const int nkt = (int)col_tiles(K);
-    bin_kernel<<<(unsigned)row_blocks(M), kBinThreads, sizeof(int32_t) * nkt, s>>>(rowptr, colidx, vals, (int)M, (int)K,
-                                                                                   nkt, t);
+    const auto kernel = !t.pos ? bin_kernel<true, false> : vals ? bin_kernel<true, true> : bin_kernel<false, true>;
+    kernel<<<(unsigned)row_blocks(M), kBinThreads, sizeof(int32_t) * nkt, s>>>(rowptr, colidx, vals, (int)M, (int)K, nkt,
+                                                                               t);
     count_launches(1);
     return check_launch("tc dense regrouping");
 }

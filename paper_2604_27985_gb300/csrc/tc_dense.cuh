@@ -24,6 +24,7 @@ struct Tiles {
     uint32_t *ent;
     int32_t *tptr;
     int32_t *bad;
+    int32_t *pos;  // ent[e]'s CSR position, or null
 };
 
 // Whether the regrouping is possible for these sizes, and whether it is worth it.
@@ -32,6 +33,7 @@ bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz);
 // ... also where the regrouping is part of every call, against the CSR kernels.
 bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz);
 
+// (vals may be null where pos is not: the words then hold no values)
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
                cudaStream_t s);
 // C = A B for N a multiple of 8 and 16-byte aligned B rows: every block of rows on the tensor
@@ -40,6 +42,17 @@ int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *val
 // err, when given, records a wait that ran out (withhold >= 0: block 0 never loads that tile).
 inline int64_t mark_count(int64_t M, int64_t N) { return row_blocks(M) * ((N + 255) / 256); }
 int launch_spmm(const SpmmProblem &p, Tiles t, int32_t *marks, int *err, int withhold, cudaStream_t s);
+
+
+// out[p] = svals[p] <X_i, Y_j> for every entry of the regrouped pattern (t.pos given): the whole
+// product of 128 X rows and 64 Y rows per tile on the tensor cores, read at the entries.  Kd of at
+// most sddmm_max_kd elements, Kd and the leading dimensions multiples of 16 bytes, 16-byte aligned X
+// and Y.  err records a wait that ran out; without it (E4M3, Kd <= 256) the blocks marked in t.bad are
+// computed again on the CUDA cores.
+inline int64_t sddmm_max_kd(bool fp8) { return fp8 ? 512 : 256; }
+bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8);
+bool sddmm_pays_unplanned(int64_t M, int64_t K, int64_t Kd, int64_t nnz);  // (E4M3 X and Y)
+int launch_sddmm(const SddmmProblem &p, Tiles t, int *err, int withhold, cudaStream_t s);
 
 }  // namespace dense
 }  // namespace gbsp

@@ -676,8 +676,8 @@ struct gbsp_plan {
     int withhold;  // see gbsp_plan_test_withhold
     gbsp_opts residual_opts;
     int residual_auto;  // the split AUTO chose for the residual at creation (0: not measured)
-    dense::Tiles tiles;  // BF16: every entry by 128 x 64 tile (tc_dense.cu), null where that does not pay
-    uint16_t *vals_full; // ... and A's values in CSR order
+    dense::Tiles tiles;  // every entry by 128 x 64 tile (tc_dense.cu), null where that does not pay
+    uint16_t *vals_full; // ... and, for BF16, A's values in CSR order
 };
 
 namespace {
@@ -713,6 +713,7 @@ void plan_free(gbsp_plan *p) {
     cudaFree(p->tiles.ent);
     cudaFree(p->tiles.tptr);
     cudaFree(p->tiles.bad);
+    cudaFree(p->tiles.pos);
     cudaFree(p->vals_full);
     cudaFree(p->err);
     delete p;
@@ -872,17 +873,21 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     }
     // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
-    if (!fp8 && by_default && dense::tiles_fit(M, K) && dense::spmm_pays(M, K, 256, p->nnz)) {
+    if (by_default && dense::tiles_fit(M, K) &&
+        (dense::spmm_pays(M, K, 256, p->nnz) || dense::sddmm_pays(M, K, 256, p->nnz, fp8))) {
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
             dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)) == GBSP_OK &&
-            dev_alloc(&p->vals_full, (size_t)p->nnz) == GBSP_OK) {
-            cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
-            GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, static_cast<const uint16_t *>(A->vals), M, K, p->tiles, s));
+            dev_alloc(&p->tiles.pos, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
+            (fp8 || dev_alloc(&p->vals_full, (size_t)p->nnz) == GBSP_OK)) {
+            if (!fp8)
+                cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
+            GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, p->vals_full, M, K, p->tiles, s));
         } else {  // no room: the plan works without
             cudaFree(p->tiles.ent);
             cudaFree(p->tiles.tptr);
             cudaFree(p->tiles.bad);
+            cudaFree(p->tiles.pos);
             cudaFree(p->vals_full);
             p->tiles = dense::Tiles{};
             p->vals_full = nullptr;
@@ -980,7 +985,7 @@ GBSP_EXPORT int gbsp_plan_execute(const gbsp_plan *p, const gbsp_dense *B, gbsp_
                     amul);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     void *marks = nullptr;
-    if (p->tiles.ent && dense::spmm_pays(p->M, p->K, N, p->nnz) &&
+    if (!fp8 && p->tiles.ent && dense::spmm_pays(p->M, p->K, N, p->nnz) &&
         scratch_alloc(&marks, sizeof(int32_t) * (size_t)dense::mark_count(p->M, N), s) == GBSP_OK) {
         SpmmProblem q{};
         q.M = (int32_t)p->M;
@@ -1082,15 +1087,38 @@ GBSP_EXPORT int gbsp_plan_sddmm(const gbsp_plan *p, const float *svals, const gb
         return fail(GBSP_ERR_ALIGN, "plan sddmm: Kd and leading dimensions multiples of %d, 16-byte aligned X and "
                                     "Y, Kd <= 512", V);
     const int kb = (int)(Kd * es / 128);
+    const bool by_default = tiles < 0;
     // the tiles pay when a dense block holds enough stored entries to outweigh gathering all
     // its 8 Y rows (measured crossover between 16 and 27 per block on 16,384^2 at 90%, Kd = 256)
     if (tiles < 0) tiles = p->nwin_tc > 0 && p->dense_nnz >= 24 * p->nblocks;
+    // whole 128 x 64 tiles (tc_dense_sddmm.cu) where the sums were the tensor cores' already (from
+    // Kd = 64 on its short parts are the more exact ones) or E4M3's, which are as exact as the CSR
+    // kernels'
+    const bool whole = by_default && p->tiles.pos && (tiles || (fp8 && Kd <= 256)) &&
+                       dense::sddmm_pays(p->M, p->K, Kd, p->nnz, fp8);
     if (tiles && p->nwin_tc > 0 && ((Kd * es) % 128 || kb < 1 || kb > 8))
         return fail(GBSP_ERR_UNSUPPORTED, "plan sddmm: tensor-core tiles need Kd a multiple of %d and at most %d",
                     128 / es, 1024 / es);
     if (p->nnz == 0 || Kd == 0) return ok();
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int st;
+    if (whole) {
+        SddmmProblem q{};
+        q.M = (int32_t)p->M;
+        q.N = (int32_t)p->K;
+        q.Kd = (int32_t)Kd;
+        q.nnz = p->nnz;
+        q.svals = svals;
+        q.X = X->data;
+        q.ldx = X->ld;
+        q.x_scale = static_cast<const float *>(X->row_scale);
+        q.Y = Y->data;
+        q.ldy = Y->ld;
+        q.y_scale = static_cast<const float *>(Y->row_scale);
+        q.out = out;
+        q.dtype = X->dtype;
+        return (st = dense::launch_sddmm(q, p->tiles, p->err, p->withhold, s)) ? st : ok();
+    }
     if (!tiles) {  // every entry through the CSR kernels on the plan's copy of the pattern
         SddmmProblem q{};
         q.M = (int32_t)p->M;

@@ -181,3 +181,92 @@ def test_dense_without_a_plan_any_column_order(gb):
     assert n == 1
     graph.replay()
     assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
+
+
+@pytest.mark.parametrize("M,K,Kd,fp8", [(2048, 2048, 64, False), (2049, 2111, 192, False), (2175, 4097, 256, False),
+                                        (2100, 2304, 128, True), (2303, 2049, 256, True), (2500, 2500, 384, False)])
+def test_dense_sddmm_integers_bit_exact(gb, M, K, Kd, fp8):  # (Kd = 384 in BF16: not the path)
+    """One launch over whole tiles: tile edges, ranges of tiles that change their row block, 1 to 4
+    accumulators, tiles past the entries loaded ahead; E4M3 with unit scales."""
+    import torch
+
+    A = matrix(M, K, 760 + Kd, 0.2, 0.45)
+    svals = gen.vals_int(A.nnz, 761)
+    X, Y = gen.dense_int(M, Kd, 762, -4, 4), gen.dense_int(K, Kd, 763, -4, 4)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(A.vals), K)
+    want, _ = oracle.sddmm(A.rowptr, A.colidx, svals, X, Y)
+    if fp8:
+        one = lambda n: torch.ones(n, device="cuda")
+        f = lambda: plan.sddmm(dev(svals), dev(oracle.e4m3_round(X)), dev(oracle.e4m3_round(Y)), x_scale=one(M), y_scale=one(K))
+    else:
+        f = lambda: plan.sddmm(dev(svals), bf16(X), bf16(Y))
+    out, n = launches(gb, f)
+    plan.check()
+    assert (n == 1) == (Kd != 384)
+    assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
+
+
+def test_dense_sddmm_random_scales_and_infinities(gb):
+    """E4M3 row scales on an E4M3 plan, padded leading dimensions; an infinity or NaN in an X or Y
+    row reaches only that row's entries."""
+    import torch
+
+    A = matrix(2400, 2600, 770, 0.2, 0.45)
+    X, Y = gen.dense_normal(2400, 256, 771), gen.dense_normal(2600, 256, 772)
+    svals = gen.dense_normal(1, A.nnz, 773)[0]
+    ones = torch.ones(A.nnz, device="cuda").to(torch.float8_e4m3fn).view(torch.uint8)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), ones, 2600, row_scale=torch.ones(2400, device="cuda"))
+    qx, sx = gb.quantize_e4m3_rows(dev(X))
+    qy, sy = gb.quantize_e4m3_rows(dev(Y))
+    wide = torch.zeros((2600, 272), dtype=torch.uint8, device="cuda")
+    wide[:, :256] = qy
+    out, n = launches(gb, lambda: plan.sddmm(dev(svals), qx, wide[:, :256], x_scale=sx, y_scale=sy))
+    plan.check()
+    dec = lambda q, s: q.view(torch.float8_e4m3fn).float().cpu().numpy().astype(np.float64) * s.cpu().numpy()[:, None]
+    ref, sc = oracle.sddmm(A.rowptr, A.colidx, svals, dec(qx, sx), dec(qy, sy))
+    assert n == 1
+    assert_within(out.cpu().numpy(), ref, sc, TOL32, "e4m3")
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(A.vals), 2600)
+    want = plan.sddmm(dev(svals), bf16(X), bf16(Y)).cpu().numpy()
+    X[130, 7], Y[700, 200] = np.nan, np.inf
+    out = plan.sddmm(dev(svals), bf16(X), bf16(Y)).cpu().numpy()
+    rows = np.repeat(np.arange(A.M), np.diff(A.rowptr))
+    hit = (rows == 130) | (A.colidx == 700)
+    assert hit.any() and np.array_equal(~np.isfinite(out), hit)
+    assert np.array_equal(out[~hit], want[~hit])
+
+
+def test_dense_sddmm_bounded_wait_reports_timeout(gb):
+    A = matrix(2048, 2048, 780, 0.2, 0.45)
+    X, Y = gen.dense_int(2048, 64, 781, -4, 4), gen.dense_int(2048, 64, 782, -4, 4)
+    svals = gen.vals_int(A.nnz, 783)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(A.vals), 2048)
+    plan.test_withhold(2)
+    plan.sddmm(dev(svals), bf16(X), bf16(Y))
+    with pytest.raises(gb.GbspError, match="TIMEOUT"):
+        plan.check()
+    plan.test_withhold(-1)
+    out = plan.sddmm(dev(svals), bf16(X), bf16(Y)).cpu().numpy()
+    plan.check()
+    assert np.array_equal(out.astype(np.float64), oracle.sddmm(A.rowptr, A.colidx, svals, X, Y)[0])
+
+
+@pytest.mark.parametrize("Kd", [128, 208, 256])
+def test_dense_sddmm_without_a_plan_any_column_order(gb, Kd):
+    """AUTO on E4M3 X and Y: the row statistics, the regrouping, the tiles and the marked rows; rows with
+    repeated or unordered columns go to the CUDA cores with their block."""
+    import torch
+
+    M, K = 10001, 2304
+    A = matrix(M, K, 790, 0.2, 0.35)
+    ci = A.colidx.copy()
+    for r in (1, 700, 701):
+        ci[A.rowptr[r]:A.rowptr[r + 1]] = ci[A.rowptr[r]:A.rowptr[r + 1]][::-1]
+    ci[A.rowptr[10000]] = ci[A.rowptr[10000] + 1]
+    svals = gen.vals_int(A.nnz, 791)
+    X, Y = gen.dense_int(M, Kd, 792), gen.dense_int(K, Kd, 793)
+    one = lambda n: torch.ones(n, device="cuda")
+    args = dev(A.rowptr), dev(ci), dev(svals), dev(oracle.e4m3_round(X)), dev(oracle.e4m3_round(Y))
+    out, n = launches(gb, lambda: gb.sddmm(*args, x_scale=one(M), y_scale=one(K)))
+    want, _ = oracle.sddmm(A.rowptr, ci, svals, X, Y)
+    assert n == 4 and np.array_equal(out.cpu().numpy().astype(np.float64), want)
