@@ -7,6 +7,8 @@ SpMM / SDDMM happens here; PyTorch only owns the memory and the stream.
 from __future__ import annotations
 
 import ctypes
+import functools
+import struct
 
 import torch
 
@@ -34,8 +36,8 @@ def _ptr(t: torch.Tensor | None) -> int | None:
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # torch.cuda.current_stream() without making a Stream object (3.0 -> 0.2 us)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -64,6 +66,37 @@ def _opts(variant="auto", validate=False, unroll=0, ctas_per_sm=0, vecs=0) -> Op
                 int(unroll), int(ctas_per_sm), int(vecs))
 
 
+# The descriptors of spmm and sddmm, whose calls are short, as packed bytes with the layout of
+# Csr, Dense and Opts (a ctypes structure takes several times as long to fill): the Python side
+# of a 1,024-row row-split SpMM takes 10.5 us instead of 21.
+_CSR, _DENSE, _OPTS = struct.Struct("qqqPPPPi0q"), struct.Struct("PqqqPi0q"), struct.Struct("5i")
+_spmm_ex, _sddmm_ex = lib["spmm_csr_ex"], lib["sddmm_csr_ex"]
+_spmm_ex.argtypes = [ctypes.c_char_p] * 4 + [ctypes.c_void_p]
+_sddmm_ex.argtypes = [ctypes.c_char_p] * 3 + [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_void_p]
+
+
+def _csr_bytes(rowptr, colidx, vals, ncols, scale=None) -> bytes:
+    if rowptr.dtype is not torch.int32 or not rowptr.is_contiguous():
+        raise TypeError("rowptr must be a contiguous int32 tensor")
+    if colidx.dtype is not torch.int32 or not colidx.is_contiguous():
+        raise TypeError("colidx must be a contiguous int32 tensor")
+    if not vals.is_contiguous():
+        raise ValueError("vals must be contiguous")
+    return _CSR.pack(rowptr.numel() - 1, ncols, colidx.numel(), _ptr(rowptr) or 0, _ptr(colidx) or 0, _ptr(vals) or 0,
+                     _ptr(scale) or 0, _dtype(vals))
+
+
+def _dense_bytes(t, scale=None) -> bytes:
+    shape = t.shape
+    return _DENSE.pack(_ptr(t) or 0, shape[0], shape[1], _ld(t), _ptr(scale) or 0, _dtype(t))
+
+
+@functools.lru_cache(maxsize=256)
+def _opts_bytes(variant, validate, unroll, ctas_per_sm, vecs) -> bytes:
+    return _OPTS.pack(VARIANTS[variant] if isinstance(variant, str) else int(variant), int(bool(validate)),
+                      int(unroll), int(ctas_per_sm), int(vecs))
+
+
 def spmm_csr(rowptr, colidx, vals, B, C, M, K, N) -> None:
     """The plain FP32 entry point (legacy default stream): C = A B, Eq. 1."""
     check(lib.spmm_csr(_ptr(rowptr), _ptr(colidx), _ptr(vals), _ptr(B), _ptr(C), int(M), int(K), int(N)))
@@ -88,10 +121,10 @@ def spmm(rowptr, colidx, vals, B, out=None, *, a_scale=None, b_scale=None, varia
     M = rowptr.numel() - 1
     if out is None:
         out = torch.empty((M, B.shape[1]), dtype=torch.float32, device=B.device)
-    A = _csr(rowptr, colidx, vals, B.shape[0], a_scale)
-    b, c = _dense(B, b_scale), _dense(out)
-    o = _opts(variant, validate, unroll, ctas_per_sm, vecs)
-    check(lib.spmm_csr_ex(ctypes.byref(A), ctypes.byref(b), ctypes.byref(c), ctypes.byref(o), _stream(stream)))
+    st = _spmm_ex(_csr_bytes(rowptr, colidx, vals, B.shape[0], a_scale), _dense_bytes(B, b_scale), _dense_bytes(out),
+                  _opts_bytes(variant, validate, unroll, ctas_per_sm, vecs), _stream(stream))
+    if st:
+        check(st)
     return out
 
 
@@ -100,11 +133,10 @@ def sddmm(rowptr, colidx, svals, X, Y, out=None, *, x_scale=None, y_scale=None, 
     """out[p] = s_p <X_i, Y_j> (Eq. 2) through sddmm_csr_ex; returns FP32 out[nnz]."""
     if out is None:
         out = torch.empty(colidx.numel(), dtype=torch.float32, device=X.device)
-    S = _csr(rowptr, colidx, svals, Y.shape[0])
-    x, y = _dense(X, x_scale), _dense(Y, y_scale)
-    o = _opts(variant, validate, vecs=vecs)
-    check(lib.sddmm_csr_ex(ctypes.byref(S), ctypes.byref(x), ctypes.byref(y), _ptr(out), ctypes.byref(o),
-                           _stream(stream)))
+    st = _sddmm_ex(_csr_bytes(rowptr, colidx, svals, Y.shape[0]), _dense_bytes(X, x_scale), _dense_bytes(Y, y_scale),
+                   _ptr(out), _opts_bytes(variant, validate, 0, 0, vecs), _stream(stream))
+    if st:
+        check(st)
     return out
 
 
