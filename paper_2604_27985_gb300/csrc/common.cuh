@@ -159,6 +159,46 @@ struct E4M3 {
     }
 };
 
+// A load of LB bytes of a row that is aligned to them, and its elements as FP32.
+template <int LB>
+struct Unit;
+template <>
+struct Unit<1> {
+    uint32_t w[1];
+    __device__ __forceinline__ void load(const void *p) { w[0] = __ldg(static_cast<const unsigned char *>(p)); }
+};
+template <>
+struct Unit<2> {
+    uint32_t w[1];
+    __device__ __forceinline__ void load(const void *p) { w[0] = __ldg(static_cast<const unsigned short *>(p)); }
+};
+template <>
+struct Unit<4> {
+    uint32_t w[1];
+    __device__ __forceinline__ void load(const void *p) { w[0] = __ldg(static_cast<const unsigned int *>(p)); }
+};
+template <>
+struct Unit<8> {
+    uint32_t w[2];
+    __device__ __forceinline__ void load(const void *p) {
+        const uint2 v = __ldg(static_cast<const uint2 *>(p));
+        w[0] = v.x;
+        w[1] = v.y;
+    }
+};
+template <class EL, int LB>
+__device__ __forceinline__ void unit_decode(const Unit<LB> &u, float (&o)[LB / (int)sizeof(typename EL::stored)]) {
+    constexpr int ES = (int)sizeof(typename EL::stored), N = LB / ES;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t w = u.w[k * ES / 4] >> (8 * (k * ES % 4));
+        if constexpr (ES == 4)
+            o[k] = __uint_as_float(w);
+        else
+            o[k] = EL::value((typename EL::stored)w);
+    }
+}
+
 // Streaming (read-once) loads: indices and values are touched once, so keep them from
 // displacing the gathered dense rows in L1 / L2.
 __device__ __forceinline__ int ld_stream(const int32_t *p) { return __ldcs(p); }
@@ -222,6 +262,14 @@ __device__ __forceinline__ int merge_search(const int32_t *rowptr, int M, int64_
     const int64_t x = lo + lane;
     const bool t = x < hi && (int64_t)__ldg(rowptr + x + 1) + x + 1 <= d;
     return (int)(lo + __popc(__ballot_sync(FULL, t)));
+}
+
+// Bytes (at most 8, a power of two, whole elements of es bytes) that divide every row of n elements
+// starting at p with leading dimension ld, and the rows' starts.
+inline int unit_bytes(const void *p, int64_t ld, int64_t n, int es) {
+    int b = 8;
+    while (b > es && (reinterpret_cast<uintptr_t>(p) % b || ld * es % b || n * es % b)) b /= 2;
+    return b;
 }
 
 // ---- launch descriptors -------------------------------------------------------------------

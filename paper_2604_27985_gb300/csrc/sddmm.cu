@@ -34,6 +34,27 @@ int run(const SddmmProblem &P, int variant, cudaStream_t s) {
     return check_launch("sddmm rowsplit");
 }
 
+template <class EL, int LB, int LPN, int T>
+int run_units_as(const SddmmProblem &P, cudaStream_t s) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sddmm_unit_kernel<EL, LB, LPN, T>, 256, 0) != cudaSuccess)
+        return check_launch("occupancy query");
+    const int nblocks = sm_count() * (per_sm < 1 ? 1 : per_sm);
+    sddmm_unit_kernel<EL, LB, LPN, T><<<dim3(nblocks), 256, 0, s>>>(P, nblocks * 8);
+    count_launches(1);
+    return check_launch("sddmm units");
+}
+
+// Four units per lane on as few lanes as cover the row (more entries per step), eight past 128.
+template <class EL, int LB>
+int run_units(const SddmmProblem &P, int units, cudaStream_t s) {
+    if (units <= 16) return run_units_as<EL, LB, 4, 4>(P, s);
+    if (units <= 32) return run_units_as<EL, LB, 8, 4>(P, s);
+    if (units <= 64) return run_units_as<EL, LB, 16, 4>(P, s);
+    if (units <= 128) return run_units_as<EL, LB, 32, 4>(P, s);
+    return run_units_as<EL, LB, 32, 8>(P, s);
+}
+
 template <class EL, int VPL>
 int by_lanes(const SddmmProblem &P, int lpn, int variant, cudaStream_t s) {
     if constexpr (VPL * EL::V > 16) {  // at most 16 elements of X_i per lane
@@ -58,6 +79,16 @@ template <class EL>
 int launch_sddmm_typed(const SddmmProblem &P, int variant, int vecs, cudaStream_t s) {
     using namespace sddmm_detail;
     if (variant == GBSP_VARIANT_SCALAR) {
+        constexpr int ES = (int)sizeof(typename EL::stored);
+        const int lx = unit_bytes(P.X, P.ldx, P.Kd, ES), ly = unit_bytes(P.Y, P.ldy, P.Kd, ES), lb = lx < ly ? lx : ly;
+        const int units = P.Kd * ES / lb;
+        if (units >= 8 && units <= 256) {
+            if constexpr (ES <= 1)
+                if (lb == 1) return run_units<EL, 1>(P, units, s);
+            if constexpr (ES <= 2)
+                if (lb == 2) return run_units<EL, 2>(P, units, s);
+            return lb == 4 ? run_units<EL, 4>(P, units, s) : run_units<EL, 8>(P, units, s);
+        }
         sddmm_scalar_kernel<EL><<<dim3((P.M + 7) / 8), 256, 0, s>>>(P);
         count_launches(1);
         return check_launch("sddmm scalar");

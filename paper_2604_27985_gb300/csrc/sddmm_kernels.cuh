@@ -348,7 +348,102 @@ __global__ void __launch_bounds__(256) sddmm_entry_kernel(const SddmmProblem P, 
         sddmm_entries<EL, LPN, VPL, true>(P, e0, e1, rc, lane);
 }
 
-// Any Kd and alignment: one lane per stored entry, plain loads.  X_i is read by all lanes
+// Any alignment, Kd of at most LPN x T units: a unit is a load of LB bytes (as many whole elements
+// as the rows' alignment and width allow).  X_i in registers; LPN lanes share an entry, lane sl of a
+// group takes units sl, sl + LPN, ..., U entries per group are loaded before any is used, and a
+// butterfly adds a group's shares.  Entries are split evenly over the warps as in the merge kernel.
+// (One lane per entry, as for the narrow Kd below, reads each Y row element by element: 30,011 x
+// 41,017, 205 entries a row, Kd = 101, FP32: 886 us, 416 now; Kd = 110 1002 -> 270; Zipf rows 1581 -> 424.)
+template <class EL, int LB, int LPN, int T>
+__device__ __forceinline__ void sddmm_unit_segment(const SddmmProblem &P, int row, int64_t p0, int64_t p1, int lane) {
+    using ST = typename EL::stored;
+    constexpr int UE = LB / (int)sizeof(ST), G = 32 / LPN, U = T >= 8 ? 2 : 4;
+    const int sl = lane % LPN, sub = lane / LPN;
+    const int units = P.Kd / UE;
+    const ST *Y = static_cast<const ST *>(P.Y);
+    // units past the row's end read its first one and are left out of the sum: no load is predicated
+    float x[T][UE];
+    int at[T];
+    bool ok[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        ok[t] = sl + LPN * t < units;
+        at[t] = ok[t] ? (sl + LPN * t) * UE : 0;
+        Unit<LB> r;
+        r.load(static_cast<const ST *>(P.X) + (int64_t)row * P.ldx + at[t]);
+        unit_decode<EL, LB>(r, x[t]);
+    }
+    const float xs = EL::dtype == GBSP_E4M3 ? __ldg(P.x_scale + row) : 1.0f;
+    int nc = 0;
+    float ns = 0.f;
+    auto load = [&](int64_t base) {  // the next 32 entries, while these are worked on
+        if (base + lane < p1) {
+            nc = ld_stream(P.colidx + base + lane);
+            ns = ld_stream(P.svals + base + lane);
+        }
+    };
+    load(p0);
+    for (int64_t base = p0; base < p1; base += 32) {
+        const int c = nc;
+        const float s = ns;
+        if (base + 32 < p1) load(base + 32);
+        const int cnt = (int)min((int64_t)32, p1 - base);
+        float mine = 0.f;  // the dot product of the chunk's entry `lane`
+        for (int q = 0; q < cnt; q += G * U) {
+            Unit<LB> y[U][T];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int cj = __shfl_sync(FULL, c, min(q + u * G + sub, cnt - 1));
+                const ST *r = Y + (int64_t)cj * P.ldy;
+#pragma unroll
+                for (int t = 0; t < T; ++t) y[u][t].load(r + at[t]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float sum = 0.f;
+#pragma unroll
+                for (int t = 0; t < T; ++t) {
+                    float o[UE];
+                    unit_decode<EL, LB>(y[u][t], o);
+#pragma unroll
+                    for (int k = 0; k < UE; ++k) sum = ok[t] ? fmaf(x[t][k], o[k], sum) : sum;
+                }
+#pragma unroll
+                for (int off = LPN / 2; off >= 1; off >>= 1) sum += __shfl_xor_sync(FULL, sum, off);
+                const int rel = lane - (q + u * G);
+                const float v = __shfl_sync(FULL, sum, (rel & (G - 1)) * LPN);
+                if (rel >= 0 && rel < G) mine = v;
+            }
+        }
+        if (lane < cnt) {
+            float r = s * mine;
+            if (EL::dtype == GBSP_E4M3) r *= xs * __ldg(P.y_scale + c);
+            __stcs(P.out + base + lane, r);
+        }
+    }
+}
+
+template <class EL, int LB, int LPN, int T>
+__global__ void __launch_bounds__(256) sddmm_unit_kernel(const SddmmProblem P, int nwarps) {
+    const int lane = threadIdx.x & 31;
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t nnz = __ldg(P.rowptr + P.M);
+    const int64_t total = (int64_t)P.M + nnz;
+    const int64_t ipw = (total + nwarps - 1) / nwarps;
+    const int64_t d0 = min((int64_t)w * ipw, total);
+    const int64_t d1 = min(d0 + ipw, total);
+    const int x0 = merge_search(P.rowptr, P.M, nnz, d0, lane);
+    const int x1 = merge_search(P.rowptr, P.M, nnz, d1, lane);
+    int64_t p = d0 - x0;
+    const int64_t y1 = d1 - x1;
+    for (int row = x0; row <= x1 && row < P.M; ++row) {
+        const int64_t e = row < x1 ? (int64_t)__ldg(P.rowptr + row + 1) : y1;
+        if (e > p) sddmm_unit_segment<EL, LB, LPN, T>(P, row, p, e, lane);
+        p = e;
+    }
+}
+
+// Any Kd and alignment (narrow ones, and those past the kernel above): one lane per stored entry, plain loads.  X_i is read by all lanes
 // of the warp at the same address (a broadcast).  Suits small Kd such as the paper's D = 2.
 template <class EL>
 __global__ void __launch_bounds__(256) sddmm_scalar_kernel(const SddmmProblem P) {

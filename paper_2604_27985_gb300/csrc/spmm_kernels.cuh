@@ -336,7 +336,99 @@ __global__ void __launch_bounds__(256) spmm_rowgroup_kernel(const SpmmProblem P)
     }
 }
 
-// Unvectorised form for any width and alignment: one warp per row, lane l owns columns
+// Any width and alignment: one warp per row, loads of LB bytes (as many whole elements as the
+// rows' alignment and width allow, UE of them), lane l owns units l, l + 32, ... of a pass of T x 32
+// units.  U entries' units are loaded before any is used and the next 32 entries while these are
+// worked on; bound by the latency of both.  30,011 x 41,017, 205 entries a row, FP32: N = 110 321 ->
+// 190 us, 101 321 -> 278, 9 221 -> 119 (the form below); Zipf rows, N = 101: 1403 -> 730.  Twice or half
+// the entries in flight: 287 / 291 at N = 101.  Each column is summed entry by entry in order,
+// whatever T, U and LB are.
+template <class EL, int LB, int T>
+__global__ void __launch_bounds__(256) spmm_unit_kernel(const SpmmProblem P) {
+    constexpr int UE = LB / (int)sizeof(typename EL::stored);
+    constexpr int U = T >= 8 ? 2 : T >= 4 ? 4 : 8;
+    const int lane = threadIdx.x & 31;
+    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (row >= P.M) return;
+    const int64_t p0 = __ldg(P.rowptr + row), p1 = __ldg(P.rowptr + row + 1);
+    const typename EL::stored *B = static_cast<const typename EL::stored *>(P.B);
+    const float sc = row_scale<EL>(P, row);
+    const int units = P.N / UE;
+    for (int u0 = 0; u0 < units; u0 += 32 * T) {
+        // lanes past the row's end read its first unit and store nothing: no load is predicated
+        float acc[T][UE];
+        int at[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            at[t] = u0 + lane + 32 * t < units ? (u0 + lane + 32 * t) * UE : 0;
+#pragma unroll
+            for (int k = 0; k < UE; ++k) acc[t][k] = 0.f;
+        }
+        int c = 0, nc = 0;
+        float a = 0.f, na = 0.f;
+        auto load = [&](int64_t base) {  // the next 32 entries, while these are worked on
+            nc = 0;
+            na = 0.f;
+            if (base + lane < p1) {
+                nc = ld_stream(P.colidx + base + lane);
+                na = coef<EL>(P, base + lane, nc);
+            }
+        };
+        load(p0);
+        for (int64_t base = p0; base < p1; base += 32) {
+            c = nc;
+            a = na;
+            if (base + 32 < p1) load(base + 32);
+            const int cnt = (int)min((int64_t)32, p1 - base);
+            int j = 0;
+            for (; j + U <= cnt; j += U) {
+                Unit<LB> raw[U][T];
+                float aj[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int cj = __shfl_sync(FULL, c, j + u);
+                    aj[u] = __shfl_sync(FULL, a, j + u);
+                    const typename EL::stored *r = B + (int64_t)cj * P.ldb;
+#pragma unroll
+                    for (int t = 0; t < T; ++t) raw[u][t].load(r + at[t]);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int t = 0; t < T; ++t) {
+                        float o[UE];
+                        unit_decode<EL, LB>(raw[u][t], o);
+#pragma unroll
+                        for (int k = 0; k < UE; ++k) acc[t][k] = fmaf(aj[u], o[k], acc[t][k]);
+                    }
+            }
+            for (; j < cnt; ++j) {
+                const int cj = __shfl_sync(FULL, c, j);
+                const float aj = __shfl_sync(FULL, a, j);
+                const typename EL::stored *r = B + (int64_t)cj * P.ldb;
+                Unit<LB> raw[T];
+#pragma unroll
+                for (int t = 0; t < T; ++t) raw[t].load(r + at[t]);
+#pragma unroll
+                for (int t = 0; t < T; ++t) {
+                    float o[UE];
+                    unit_decode<EL, LB>(raw[t], o);
+#pragma unroll
+                    for (int k = 0; k < UE; ++k) acc[t][k] = fmaf(aj, o[k], acc[t][k]);
+                }
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            float *dst = P.C + (int64_t)row * P.ldc + (int64_t)(u0 + lane + 32 * t) * UE;
+            if (u0 + lane + 32 * t < units)
+#pragma unroll
+                for (int k = 0; k < UE; ++k) dst[k] = acc[t][k] * sc;
+        }
+    }
+}
+
+// ... for rows of a few entries, which the units' registers (fewer warps per SM) do not help: one warp per row, lane l owns columns
 // l, l + 32, l + 64, l + 96 of a 128-column pass.
 template <class EL>
 __global__ void __launch_bounds__(256) spmm_scalar_kernel(const SpmmProblem P) {
