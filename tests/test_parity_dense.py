@@ -118,6 +118,28 @@ def test_dense_infinities_and_nan_stay_in_their_rows(gb):
     assert np.array_equal(C.astype(np.float64), want)
 
 
+def test_dense_plan_under_capture(gb):
+    """A plan's executions replay from a CUDA graph (their scratch is the graph's)."""
+    import torch
+
+    A = matrix(2048, 2048, 725)
+    vals = gen.vals_int(A.nnz, 726)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(vals), 2048)
+    b, out = torch.zeros((2048, 128), dtype=torch.bfloat16, device="cuda"), torch.empty((2048, 128), device="cuda")
+    plan.execute(b, out=out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        _, n = launches(gb, lambda: plan.execute(b, out=out))
+    assert n == 2
+    for seed in (727, 728):
+        B = gen.dense_int(2048, 128, seed)
+        b.copy_(bf16(B))
+        graph.replay()
+        want, _ = oracle.spmm(A.rowptr, A.colidx, vals, B)
+        assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
+    plan.check()
+
+
 def test_dense_bounded_wait_reports_timeout(gb):
     """A tile whose B rows never arrive: the waits give up, the plan reports the timeout, and
     the block's rows are computed again on the CUDA cores."""
