@@ -209,6 +209,10 @@ int gbsp_spmm_sddmm_host(const int32_t *rowptr, const int32_t *colidx, const flo
  * of the window's condensed 16 x Kc tile with the Kc gathered rows of B (FP32 accumulation
  * in tensor memory), added into C.  The plan keeps its own device copy of everything it
  * needs; A (and its row scales) may be freed after creation.
+ * With threshold < 1 and default residual_opts, a BF16 plan of a matrix with a few percent of
+ * entries and more runs whole 128 x 64 tiles on the tensor cores instead where that is faster
+ * (the library decides per execution; row blocks whose result is not finite are computed again
+ * from the stored entries only).
  * BF16 (kind::f16): A->dtype BF16; at execution B BF16 (K x N).
  * E4M3 (kind::f8f6f4): A->dtype E4M3 with A->row_scale (M floats, value = s_i * q);
  * at execution B E4M3 with B->row_scale (K floats, value = t_k * q).  A scale along the
@@ -245,7 +249,8 @@ int gbsp_plan_execute(const gbsp_plan *plan, const gbsp_dense *B, gbsp_dense *C,
  * (GBSP_ERR_UNSUPPORTED).  tiles: 1 uses the tiles as above, 0 runs every entry through the
  * CSR kernels on the plan's copy of the pattern, < 0 chooses: the tiles when the dense
  * blocks average at least 24 stored entries (below that, gathering a block's 8 Y rows costs
- * more than its entries' rows).  Asynchronous; waits are bounded as in gbsp_plan_execute
+ * more than its entries' rows), and of a plan made with threshold < 1, whole 128 x 64 tiles where
+ * that is faster and no less exact.  Asynchronous; waits are bounded as in gbsp_plan_execute
  * (see gbsp_plan_check). */
 int gbsp_plan_sddmm(const gbsp_plan *plan, const float *svals, const gbsp_dense *X, const gbsp_dense *Y, float *out,
                     int32_t tiles, void *stream);
