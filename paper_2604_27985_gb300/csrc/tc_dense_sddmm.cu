@@ -406,7 +406,10 @@ int encode(const void *data, int64_t rows, int64_t cols, int64_t ld, bool fp8, i
 // CSR kernels alone, 12 / 16 / 24 ps per entry at Kd = 64 / 128 / 256.  On 16,384^2 the lines
 // cross near 7.5% / 5.5% / 3.7% of entries.
 bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8) {
-    if (M < 2048 || K < 2048 || Kd > sddmm_max_kd(fp8) || (double)nnz < 0.03 * (double)M * (double)K) return false;
+    // (rows of at least one 128-byte block: a copy's box does not pass the row's width)
+    if (M < 2048 || K < 2048 || Kd > sddmm_max_kd(fp8) || Kd < (fp8 ? 128 : 64) ||
+        (double)nnz < 0.03 * (double)M * (double)K)
+        return false;
     const double tile = 0.95 * (double)(row_blocks(M) * col_tiles(K)) / (double)(sm_count() > 0 ? sm_count() : 1);
     return tile + 8.0 < 0.9e-6 * (double)nnz * (8.0 + 0.062 * (double)Kd);
 }
@@ -417,7 +420,7 @@ bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8) {
 // (8.0e-8 against 6.1e-8).  The E4M3 CSR kernel is bound by its conversions: 16 / 30 ps per entry at
 // Kd = 128 / 256.
 bool sddmm_pays_unplanned(int64_t M, int64_t K, int64_t Kd, int64_t nnz) {
-    if (M < 2048 || K < 2048 || Kd > 256 || (double)nnz < 0.03 * (double)M * (double)K) return false;
+    if (M < 2048 || K < 2048 || Kd > 256 || Kd < 128 || (double)nnz < 0.03 * (double)M * (double)K) return false;
     const int64_t sms = sm_count() > 0 ? sm_count() : 1, nb = row_blocks(M);
     const double tile = 0.95 * (double)(nb * col_tiles(K)) / (double)sms;
     const double bins = (double)((nb + sms - 1) / sms) * 0.6e-3 * (double)nnz / (double)nb;
