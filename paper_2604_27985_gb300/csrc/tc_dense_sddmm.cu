@@ -11,11 +11,11 @@
 // The tensor core's accumulation is not rounded to nearest, so Kd is cut into four parts with an
 // accumulator each, added in FP32: error against 64 bits at Kd = 256 in BF16 8.1e-8 (the 16 x 8
 // blocks' one accumulator and their CSR residual together 1.7e-7, the CSR kernel 6.1e-8), in
-// E4M3 4.6e-8 (4.7e-8, 4.5e-8).
+// E4M3 3.0e-8 (4.7e-8, 4.5e-8), where value and scales are applied with one rounding.
 //
 // 16,384^2 at 90%, half in dense blocks, Kd = 256: BF16 on a plan 637 -> 215 us, where the MMAs alone
 // (N = 64 reads A's rows from shared memory for little work: 92 clocks each) take 152; E4M3 without
-// a plan 803 -> 428 with the regrouping's 130.  On the way: 328 us with the tile coordinates by
+// a plan 804 -> 447 with the regrouping's 130.  On the way: 328 us with the tile coordinates by
 // 64-bit division in every warp, 245 without.
 #include <mutex>
 
@@ -71,6 +71,16 @@ __device__ __forceinline__ void add(float (&x)[16], const float (&y)[16]) {
         x[j] = v.x;
         x[j + 1] = v.y;
     }
+}
+
+// (v + ev) * x * y rounded once, ev being the rounding error of v: the three roundings of v * (x * y)
+// are most of the E4M3 form's error (16,384^2 at 90%, Kd = 256: 4.57e-8 with them, 3.0e-8 so; the CSR
+// kernel has 4.55e-8, and the whole call takes 447 us against 439).  v * (x * y) itself where something is
+// not finite and for a zero's sign.
+__device__ __forceinline__ float scaled(float v, float ev, float x, float y) {
+    const float p = __fmul_rn(x, y), plain = __fmul_rn(v, p);
+    const float exact = __fmaf_rn(v, p, __fmaf_rn(v, __fmaf_rn(x, y, -p), __fmul_rn(ev, p)));
+    return fabsf(exact) > 0.f && fabsf(exact) < __int_as_float(0x7f800000) ? exact : plain;
 }
 
 template <int V>
@@ -233,10 +243,11 @@ __global__ void __launch_bounds__(kThreads, 1) sddmm_kernel(const __grid_constan
             if (lane == 0) mbar_arrive(&dfree[g]);
             ok = bar_all(1 + g, kGroupThreads, ok);  // every row of the tile is staged
             auto emit = [&](uint32_t w, int p, float sv) {
-                float v = sv * *reinterpret_cast<const float *>(st + (w & 0xffffu) * 2);
+                const float d = *reinterpret_cast<const float *>(st + (w & 0xffffu) * 2);
+                float v = __fmul_rn(sv, d);
                 if (FP8) {
                     const int r = (w >> 7) & 127, c = (((w >> 4 ^ r) & 7) << 3) + ((w >> 1) & 7);
-                    v *= own[r] * own[kRows + c];
+                    v = scaled(v, __fmaf_rn(sv, d, -v), own[r], own[kRows + c]);
                 }
                 a.out[p] = v;
             };
@@ -415,8 +426,8 @@ bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8) {
 }
 
 // ... with the regrouping in every call (0.6 ns per entry of a block of rows, a wave of blocks at a
-// time).  E4M3 only: at Kd <= 256 its error is the CSR kernel's (4.57e-8 against 4.55e-8 on
-// 16,384^2 at 90%, Kd = 256; 4.52e-8 both at 128), BF16's four steps per part have the larger one
+// time).  E4M3 only: at Kd <= 256 its error is below the CSR kernel's (3.0e-8 against 4.55e-8 on
+// 16,384^2 at 90%, Kd = 256), BF16's four steps per part have the larger one
 // (8.0e-8 against 6.1e-8).  The E4M3 CSR kernel is bound by its conversions: 16 / 30 ps per entry at
 // Kd = 128 / 256.
 bool sddmm_pays_unplanned(int64_t M, int64_t K, int64_t Kd, int64_t nnz) {

@@ -292,3 +292,24 @@ def test_dense_sddmm_without_a_plan_any_column_order(gb, Kd):
     out, n = launches(gb, lambda: gb.sddmm(*args, x_scale=one(M), y_scale=one(K)))
     want, _ = oracle.sddmm(A.rowptr, ci, svals, X, Y)
     assert n == 4 and np.array_equal(out.cpu().numpy().astype(np.float64), want)
+
+
+@pytest.mark.parametrize("Kd", [128, 208, 256])
+def test_dense_sddmm_scales_and_value_round_once(gb, Kd):
+    """E4M3 with whole-number dots (exact): value times dot times both scales is within half a unit in
+    the last place, 2^-24 relative, and terms of 2^-47 of the exact product."""
+    import torch
+
+    M, K = 10001, 2304
+    A = matrix(M, K, 795, 0.2, 0.35)
+    svals = gen.dense_normal(1, A.nnz, 796)[0]
+    X, Y = gen.dense_int(M, Kd, 797), gen.dense_int(K, Kd, 798)
+    sx = torch.rand(M, device="cuda", generator=torch.Generator("cuda").manual_seed(1)) + 0.5
+    sy = torch.rand(K, device="cuda", generator=torch.Generator("cuda").manual_seed(2)) + 0.5
+    args = dev(A.rowptr), dev(A.colidx), dev(svals), dev(oracle.e4m3_round(X)), dev(oracle.e4m3_round(Y))
+    out, n = launches(gb, lambda: gb.sddmm(*args, x_scale=sx, y_scale=sy))
+    f64 = lambda s: s.cpu().numpy().astype(np.float64)
+    dots, _ = oracle.sddmm(A.rowptr, A.colidx, np.ones(A.nnz), X, Y)
+    want = dots * svals * np.repeat(f64(sx), np.diff(A.rowptr)) * f64(sy)[A.colidx]
+    assert n == 4
+    assert np.all(np.abs(f64(out) - want) <= 2.0**-24 * (1 + 1e-6) * np.abs(want))
