@@ -598,6 +598,8 @@ int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *val
 }
 
 int launch_spmm(const SpmmProblem &p, Tiles t, int32_t *marks, int *err, int withhold, cudaStream_t s) {
+    if (p.N % 8 || p.ldb % 8 || !aligned16(p.B))
+        return fail(GBSP_ERR_ALIGN, "tc dense: N and ld multiples of 8 and a 16-byte aligned B");
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(GBSP_ERR_CUDA, "tc dense: cuTensorMapEncodeTiled is not available");
     CUtensorMap map;

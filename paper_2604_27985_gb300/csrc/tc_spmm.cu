@@ -984,8 +984,12 @@ GBSP_EXPORT int gbsp_plan_execute(const gbsp_plan *p, const gbsp_dense *B, gbsp_
                                           "of %d and a 16-byte aligned B",
                     amul);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // (whole tiles store groups of 8 columns and copy B in 16-byte pieces; a plan without dense windows takes
+    // any other B on the CSR kernels below)
+    const bool whole = !fp8 && p->tiles.ent && N % 8 == 0 && B->ld % 8 == 0 && aligned16(B->data) &&
+                       dense::spmm_pays(p->M, p->K, N, p->nnz);
     void *marks = nullptr;
-    if (!fp8 && p->tiles.ent && dense::spmm_pays(p->M, p->K, N, p->nnz) &&
+    if (whole &&
         scratch_alloc(&marks, sizeof(int32_t) * (size_t)dense::mark_count(p->M, N), s) == GBSP_OK) {
         SpmmProblem q{};
         q.M = (int32_t)p->M;

@@ -158,6 +158,31 @@ def test_dense_bounded_wait_reports_timeout(gb):
     assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
 
 
+@pytest.mark.parametrize("N,ld,off", [(208, 208, 0), (204, 204, 0), (204, 208, 0), (200, 208, 4), (200, 204, 0)])
+def test_dense_plan_without_dense_windows_takes_any_operand(gb, N, ld, off):
+    """Columns congruent to the row modulo 11: 9% of entries and no 16 x 8 block of 14.  Such a plan
+    takes any width, leading dimension and alignment of B; whole tiles only those of 16 bytes."""
+    import torch
+
+    M, K = 12000, 3400
+    rows = [np.arange(r % 11, K, 11, dtype=np.int32) for r in range(11)]
+    rowptr = np.concatenate([[0], np.cumsum([rows[r % 11].size for r in range(M)])]).astype(np.int32)
+    colidx = np.concatenate([rows[r % 11] for r in range(M)])
+    vals, B = gen.vals_int(colidx.size, 734), gen.dense_int(K, N, 735)
+    plan = gb.TcPlan(dev(rowptr), dev(colidx), bf16(vals), K)
+    assert plan.info()["dense_windows"] == 0
+    flat = torch.zeros(off + K * ld, dtype=torch.bfloat16, device="cuda")
+    b = flat[off:].view(K, ld)[:, :N]
+    b.copy_(bf16(B))
+    full = torch.full((M + 1, N + 4), 7.0, device="cuda")
+    C, n = launches(gb, lambda: plan.execute(b, out=full[:M, :N]))
+    plan.check()
+    want, _ = oracle.spmm(rowptr, colidx, vals, B)
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), want)
+    assert bool((full[:, N:] == 7.0).all()) and bool((full[M] == 7.0).all())
+    assert (n == 2) == (N == 208)  # the tile kernel and the marked rows
+
+
 def launches(gb, f):
     before = gb.launch_count()
     out = f()
