@@ -983,11 +983,15 @@ GBSP_EXPORT int gbsp_plan_execute(const gbsp_plan *p, const gbsp_dense *B, gbsp_
         return fail(GBSP_ERR_UNSUPPORTED, "plan execute: tensor-core tiles need 64 <= N <= 512, N and ld multiples "
                                           "of %d and a 16-byte aligned B",
                     amul);
+    if (B->cols > 0 && ((B->rows > 0 && !B->data) || (C->rows > 0 && !C->data)))
+        return fail(GBSP_ERR_INVALID_ARG, "plan execute: null B / C data");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // (whole tiles store groups of 8 columns and copy B in 16-byte pieces; a plan without dense windows takes
     // any other B on the CSR kernels below)
     const bool whole = !fp8 && p->tiles.ent && N % 8 == 0 && B->ld % 8 == 0 && aligned16(B->data) &&
                        dense::spmm_pays(p->M, p->K, N, p->nnz);
+    if (whole && injected_fault() == 2)
+        return fail(GBSP_ERR_CUDA, "plan execute: injected launch failure (GBSP_FAULT=launch)");
     void *marks = nullptr;
     if (whole &&
         scratch_alloc(&marks, sizeof(int32_t) * (size_t)dense::mark_count(p->M, N), s) == GBSP_OK) {

@@ -183,6 +183,22 @@ def test_dense_plan_without_dense_windows_takes_any_operand(gb, N, ld, off):
     assert (n == 2) == (N == 208)  # the tile kernel and the marked rows
 
 
+def test_dense_plan_refuses_null_operands(gb):
+    """Null B or C data is an argument error that launches nothing, as on the CSR kernels."""
+    import ctypes
+
+    from paper_2604_27985_gb300 import ops
+
+    A = matrix(2048, 2048, 736)
+    plan = gb.TcPlan(dev(A.rowptr), dev(A.colidx), bf16(gen.vals_int(A.nnz, 737)), 2048)
+    b = bf16(gen.dense_int(2048, 64, 738))
+    for null in (0, 1):
+        d = [ops._dense(b), ops._dense(b.float())]
+        d[null].data = None
+        st, n = launches(gb, lambda: ops.lib.gbsp_plan_execute(plan._h, *(ctypes.byref(x) for x in d), None))
+        assert st == -1 and n == 0
+
+
 def launches(gb, f):
     before = gb.launch_count()
     out = f()
