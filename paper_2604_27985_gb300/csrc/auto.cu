@@ -83,12 +83,14 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const int32_t *__restric
             out->empty = atomicAdd(&acc->empty, 0ull);
             out->maxlen = atomicMax(&acc->maxlen, 0u);
             out->nnz = rowptr[M];
-            __threadfence_system();  // the host reads the counters once it has seen the token
-            *(volatile unsigned int *)&out->token = token;
             acc->sumsq = 0;
             acc->empty = 0;
             acc->maxlen = 0;
             acc->blocks_done = 0;
+            // The host that has seen the token reads the counters and may queue the next measurement into acc
+            // on any stream: the token is the last store of this one
+            __threadfence_system();
+            *(volatile unsigned int *)&out->token = token;
         }
     }
 }

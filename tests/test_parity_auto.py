@@ -251,3 +251,27 @@ def test_auto_sddmm_keeps_the_row_split_for_a_y_past_l2(gb):
     gb.auto_forget()
     for yb, rb in ((512 << 20, 512), (512 << 20, 128), (64 << 20, 512)):
         assert gb.auto_choice(rp, A.K, ci, op="sddmm", b_bytes=yb, row_bytes=rb)[0] == "rowsplit"
+
+
+def test_auto_measurements_from_two_streams(gb):
+    """Calls on one pattern from two streams in turn: every measurement counts the whole pattern, and a
+    pattern put in its place is still measured and adopted afterwards."""
+    import torch
+
+    A, P = gen.csr_uniform(8192, 8192, 0.995, seed=660), gen.csr_powerlaw(8192, 8192, 0.995, seed=661)
+    rp, ci = dev(A.rowptr), dev(A.colidx)
+    want = lambda m: {"rows": m.M, "nnz": m.nnz, "sum_sq_lengths": int((np.diff(m.rowptr).astype(np.int64) ** 2).sum()),
+                      "max_length": int(np.diff(m.rowptr).max()), "empty_rows": int((np.diff(m.rowptr) == 0).sum())}
+    gb.auto_forget()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for k in range(400):
+        _, st = gb.auto_choice(rp, A.K, ci, stream=streams[k % 2])
+        assert st == want(A), k
+        if k % 50 == 49:
+            torch.cuda.synchronize()
+    rp.copy_(dev(P.rowptr))
+    for k in range(4):
+        torch.cuda.synchronize()
+        _, st = gb.auto_choice(rp, A.K, ci, stream=streams[k % 2])
+    assert st == want(P)
