@@ -130,7 +130,11 @@ void settle(const Entry &e) {
     const auto t0 = std::chrono::steady_clock::now();
     while (e.pending && !arrived(e))
         if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(2)) {
+            int dev = e.device;  // (the caller's device need not be the entry's)
+            cudaGetDevice(&dev);
+            cudaSetDevice(e.device);
             cudaDeviceSynchronize();
+            cudaSetDevice(dev);
             return;
         }
 }
