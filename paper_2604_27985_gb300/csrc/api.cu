@@ -262,7 +262,7 @@ GBSP_EXPORT int spmm_csr_ex(const gbsp_csr *A, const gbsp_dense *B, gbsp_dense *
         const int64_t rb = B->cols * elem_bytes(B->dtype);
         if (vec && (st = auto_choice(*A, kOpSpmm, B->rows * rb, rb, s, &variant, nullptr))) return st;
         if (variant == GBSP_VARIANT_ROWSPLIT && !o.vecs && !o.unroll && A->dtype == GBSP_BF16 && A->nnz > 0 &&
-            dense::tiles_fit(A->rows, A->cols) &&
+            dense::tiles_fit(A->rows, A->cols, A->nnz) &&
             dense::spmm_pays_unplanned(A->rows, A->cols, B->cols, A->nnz)) {
             bool done = false;
             if ((st = spmm_dense(*A, *B, *C, s, &done))) return st;
@@ -314,7 +314,8 @@ GBSP_EXPORT int sddmm_csr_ex(const gbsp_csr *S, const gbsp_dense *X, const gbsp_
         const int64_t rb = Y->cols * elem_bytes(Y->dtype);
         if (vec && (st = auto_choice(*S, kOpSddmm, Y->rows * rb, rb, s, &variant, nullptr))) return st;
         if (variant == GBSP_VARIANT_ROWSPLIT && !o.vecs && X->dtype == GBSP_E4M3 && S->nnz > 0 &&
-            dense::tiles_fit(S->rows, S->cols) && dense::sddmm_pays_unplanned(S->rows, S->cols, X->cols, S->nnz)) {
+            dense::tiles_fit(S->rows, S->cols, S->nnz) &&
+            dense::sddmm_pays_unplanned(S->rows, S->cols, X->cols, S->nnz)) {
             bool done = false;
             if ((st = sddmm_dense(*S, *X, *Y, out, s, &done))) return st;
             if (done) return ok();

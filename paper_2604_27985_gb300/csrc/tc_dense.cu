@@ -543,8 +543,9 @@ int launch_nt(const CUtensorMap &map, const Args &a, int nb, cudaStream_t s) {
 
 }  // namespace
 
-bool tiles_fit(int64_t M, int64_t K) {
-    return M > 0 && K > 0 && col_tiles(K) <= kMaxTiles && row_blocks(M) * (col_tiles(K) + 1) < (1LL << 31);
+bool tiles_fit(int64_t M, int64_t K, int64_t nnz) {
+    return M > 0 && K > 0 && nnz < (1LL << 31) - 4096 && col_tiles(K) <= kMaxTiles &&
+           row_blocks(M) * (col_tiles(K) + 1) < (1LL << 31);
 }
 
 

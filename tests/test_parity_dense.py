@@ -246,6 +246,26 @@ def test_dense_without_a_plan_any_column_order(gb):
     assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
 
 
+def test_entries_near_2_to_the_31_stay_on_the_csr_kernels(gb):
+    """Whole tiles count entries in 32 bits and look past the last one: 1,000 entries short of 2^31 - 1
+    AUTO takes the row split (the statistics and one launch).  Full rows of ones: column sums."""
+    import torch
+
+    n = 46341
+    nnz = 2**31 - 1 - 1000
+    last = nnz - (n - 1) * n
+    rowptr = torch.arange(n + 1, device="cuda", dtype=torch.int64) * n
+    rowptr[n] = nnz
+    colidx = torch.arange(n, device="cuda", dtype=torch.int32).repeat(n)[:nnz]
+    vals = torch.ones(nnz, device="cuda", dtype=torch.bfloat16)
+    B = gen.dense_int(n, 128, 756)
+    C, k = launches(gb, lambda: gb.spmm(rowptr.int(), colidx, vals, bf16(B)))
+    C = C.cpu().numpy().astype(np.float64)
+    assert np.array_equal(C[:-1], np.broadcast_to(B.sum(0, dtype=np.float64), (n - 1, 128)))
+    assert np.array_equal(C[-1], B[:last].sum(0, dtype=np.float64))
+    assert k == 2
+
+
 @pytest.mark.parametrize("M,K,Kd,fp8", [(2048, 2048, 64, False), (2049, 2111, 192, False), (2175, 4097, 256, False),
                                         (2100, 2304, 128, True), (2303, 2049, 256, True), (2500, 2500, 384, False)])
 def test_dense_sddmm_integers_bit_exact(gb, M, K, Kd, fp8):  # (Kd = 384 in BF16: not the path)
