@@ -196,12 +196,14 @@ int spmm_dense(const gbsp_csr &A, const gbsp_dense &B, const gbsp_dense &C, cuda
     const int64_t nent = (dense::ent_count(A.nnz) + 3) & ~3LL, nb = dense::row_blocks(A.rows);
     const int64_t nptr = nb * (dense::col_tiles(A.cols) + 1);
     void *w = nullptr;
-    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(nent + nptr + nb + dense::mark_count(A.rows, B.cols)), s))
+    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(nent + nptr + 2 * nb + dense::mark_count(A.rows, B.cols)), s))
         return GBSP_OK;
     int32_t *i32 = static_cast<int32_t *>(w);
-    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + nent, i32 + nent + nptr, nullptr};
-    int st = dense::launch_bin(A.rowptr, A.colidx, static_cast<const uint16_t *>(A.vals), A.rows, A.cols, t, s);
-    if (!st) st = dense::launch_spmm(spmm_problem(A, B, C), t, i32 + nent + nptr + nb, nullptr, -1, s);
+    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + nent, i32 + nent + nptr, i32 + nent + nptr + nb,
+                         nullptr};
+    int st = dense::launch_bin(A.rowptr, A.colidx, static_cast<const uint16_t *>(A.vals), A.rows, A.cols, A.nnz, t,
+                               s);
+    if (!st) st = dense::launch_spmm(spmm_problem(A, B, C), t, i32 + nent + nptr + 2 * nb, nullptr, -1, s);
     scratch_free(w, s);
     *done = true;
     return st;
@@ -215,10 +217,11 @@ int sddmm_dense(const gbsp_csr &S, const gbsp_dense &X, const gbsp_dense &Y, flo
     const int64_t nent = (dense::ent_count(S.nnz) + 3) & ~3LL, nb = dense::row_blocks(S.rows);
     const int64_t nptr = nb * (dense::col_tiles(S.cols) + 1);
     void *w = nullptr;
-    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(2 * nent + nptr + nb), s)) return GBSP_OK;
+    if (scratch_alloc(&w, sizeof(int32_t) * (size_t)(2 * nent + nptr + 2 * nb), s)) return GBSP_OK;
     int32_t *i32 = static_cast<int32_t *>(w);
-    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + 2 * nent, i32 + 2 * nent + nptr, i32 + nent};
-    int st = dense::launch_bin(S.rowptr, S.colidx, nullptr, S.rows, S.cols, t, s);
+    const dense::Tiles t{reinterpret_cast<uint32_t *>(w), i32 + 2 * nent, i32 + 2 * nent + nptr,
+                         i32 + 2 * nent + nptr + nb, i32 + nent};
+    int st = dense::launch_bin(S.rowptr, S.colidx, nullptr, S.rows, S.cols, S.nnz, t, s);
     if (!st) st = dense::launch_sddmm(sddmm_problem(S, X, Y, out), t, nullptr, -1, s);
     scratch_free(w, s);
     *done = true;

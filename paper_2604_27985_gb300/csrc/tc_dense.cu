@@ -7,12 +7,14 @@
 // shared memory (already in the MMA's K-major 128-byte-swizzled image), loads the 64 B rows by
 // TMA and multiplies with tcgen05.mma (M = 128 rows, N = the features, K = 64).
 //
-// The products of BF16 values are exact; the tensor core's accumulation is not rounded to
-// nearest, and its error grows with the number of steps.  So an accumulator in TMEM runs over
-// 512 columns only, and the worker warps add it to FP32 sums in registers, two accumulators
-// alternating.  Error against 64 bits on 16,384^2 at 90%, uniform: 1.53e-7 with 256 columns per
-// accumulator (where the register sums' rounding dominates), 1.28e-7 with 512, 1.50e-7 with
-// 1,024; the CSR kernel has 2.0e-7 (N = 256), the 16 x 8 blocks over all columns 9.7e-7.
+// The products of BF16 values are exact; the tensor core cuts each at the accumulator's last bit, so its
+// error grows with the entries that one accumulator takes.  So an accumulator in TMEM runs over at most
+// 512 columns, in a block of rows with more entries there than suit it (sum_limit) over 256, 128 or
+// 64, and the worker warps add it to FP32 sums in registers, two accumulators alternating.  Error
+// against 64 bits on 16,384^2 at 90%, uniform: 1.53e-7 with 256 columns per accumulator (where the
+// register sums' rounding dominates), 1.28e-7 with 512, 1.50e-7 with 1,024; the CSR kernel has 2.0e-7
+// (N = 256), the 16 x 8 blocks over all columns 9.7e-7.  With values and B of one sign an accumulator
+// of e entries a row is 1.9e-9 e too small: 512 columns at 10% / 40% of entries 9.6e-8 / 4.5e-7.
 //
 // The expanded zeros meet B's values: an infinity or NaN in any B row makes NaN in every row
 // of C.  Every accumulated value is tested at the end, and a block with one that is not finite
@@ -50,12 +52,16 @@ using namespace gbsp::tc;
 constexpr int kColBits = 6;  // log2(kCols)
 static_assert(1 << kColBits == kCols, "tiles of 64 columns");
 constexpr int kBinThreads = 1024;
+constexpr int kLogChunk = 3;  // log2 of the tiles of a TMEM accumulator at most: 512 columns of A
+constexpr int kChunk = 1 << kLogChunk;
 constexpr int kMaxTiles = 8 * 1024;  // one shared-memory counter per tile of a row block
 
 // Entries [p0, p1) of a row, U chunks of 32 at a time with the next U chunks' loads in flight:
 // f(columns, values, first entry of the first chunk, whether every lane holds an entry).  Lanes past
 // p1 hold column kNone.
 constexpr int kNone = 0x7fffffff;
+template <int V>
+struct Int { static constexpr int value = V; };
 struct true_t { static constexpr bool value = true; };
 struct false_t { static constexpr bool value = false; };
 template <int U, bool VALS, class F>
@@ -113,15 +119,15 @@ template <bool VALS, bool POS>
 __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restrict__ rowptr,
                                                           const int32_t *__restrict__ colidx,
                                                           const uint16_t *__restrict__ vals, int M, int K, int nkt,
-                                                          Tiles t) {
+                                                          Tiles t, int2 limit) {
     constexpr int U = 4;
     extern __shared__ int32_t cnt[];  // nkt counters, then cursors
     __shared__ int32_t warp_sum[32];
-    __shared__ int32_t carry;
+    __shared__ int32_t carry, over;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = blockIdx.x, r0 = b * kRows, r1 = min(r0 + kRows, M);
     for (int i = tid; i < nkt; i += kBinThreads) cnt[i] = 0;
-    if (tid == 0) carry = 0;
+    if (tid == 0) carry = over = 0;
     __syncthreads();
     bool good = true;
     for (int r = r0 + warp; r < r1; r += kBinThreads / 32) {
@@ -172,9 +178,23 @@ __global__ void __launch_bounds__(kBinThreads) bin_kernel(const int32_t *__restr
         if (tid == kBinThreads - 1) carry = before + x;
         __syncthreads();
     }
+    // bit k of over: some 2^(k + 1) tiles (from a multiple of that on) hold more entries than the narrow
+    // form's limit; bit 3 + k: ... the wide form's
+    auto first = [&](int i) { return i < nkt ? cnt[i] : start + carry; };
+    int mine = 0;
+    for (int i = 2 * tid; i < nkt; i += 2 * kBinThreads)
+#pragma unroll
+        for (int k = 0; k < kLogChunk; ++k) {
+            const int held = i % (2 << k) == 0 ? first(i + (2 << k)) - first(i) : 0;
+            mine |= (held > limit.x) << k | (held > limit.y) << (kLogChunk + k);
+        }
+    if (mine) atomicOr(&over, mine);
+    __syncthreads();
     if (tid == 0) {
         tp[nkt] = start + carry;
         t.bad[b] = bad ? 1 : 0;
+        const int narrow = over & (kChunk - 1), wide = over >> kLogChunk;  // (the lowest bit: how often 512 columns are halved)
+        t.chunk[b] = (narrow ? __ffs(narrow) - 1 : kLogChunk) | (wide ? __ffs(wide) - 1 : kLogChunk) << 4;
     }
     if (bad) return;
     const unsigned upto = FULL >> (31 - lane), beyond = ~upto;
@@ -212,8 +232,6 @@ constexpr int kGroups = 4;                      // groups of four warps that exp
 constexpr int kWorkers = 4 * kGroups;
 constexpr int kThreads = (kWorkers + 2) * 32;   // + one warp that copies, one that issues MMAs
 constexpr int kATileBytes = kRows * kCols * 2;  // 16 KB
-constexpr int kTurns = 2;                       // turns of all groups per TMEM accumulator
-constexpr int kChunk = kTurns * kGroups;        // its tiles: 512 columns of A
 constexpr int kSlot = 1072;                     // words of an entry slot (any more come from global memory)
 constexpr int kAhead = 3;                       // turns between the L2 prefetch of a tile's entries and their copy
 
@@ -276,7 +294,7 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_kernel(const __grid_constant
         if (tid == 0) a.marks[blockIdx.y * gridDim.x + b] = 1;
         return;
     }
-    const int nst = a.nkt, nchunks = (nst + kChunk - 1) / kChunk;
+    const int nst = a.nkt, lg = __ldg(a.t.chunk + b) >> (NT == 256 ? 4 : 0) & 15;  // log2 of an accumulator's tiles
     const int32_t *tp = a.t.tptr + (int64_t)b * (a.nkt + 1);
     const int n0 = blockIdx.y * NT;
 
@@ -407,10 +425,12 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_kernel(const __grid_constant
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[i % SB]);
-            // the previous accumulator: complete before this stage's turn comes again
-            if (turn / kTurns > drained) drain(drained++);
+            // Accumulators that ended before this tile need nothing more of this group.  (The MMAs of tile i wait
+            // for all groups to drain the accumulator before last, which ended by tile i - 2: a group reaches
+            // that after it expanded a tile up to i + 2, for which it needs the MMAs of tiles up to i - 2.)
+            while (ok && (drained + 1) << lg <= i) drain(drained++);
         }
-        while (ok && drained < nchunks) drain(drained++);
+        while (ok && drained << lg < nst) drain(drained++);
         if (!ok) {
             *failed = 1;
             if (t == 0)  // copies still on their way land before the CTA can leave
@@ -445,21 +465,31 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_kernel(const __grid_constant
         const uint64_t ad0 = smem_desc(smem_u32(smem), 16, 1024), bd0 = smem_desc(smem_u32(bring), kCols * 128, 1024);
         const bool one = elect_one();
         bool ok = true;
-        for (int i = 0; i < nst; ++i) {
-            const int s = i % SB, c = i / kChunk;
-            if (i % kChunk == 0 && c >= 2) ok = __all_sync(FULL, mbar_wait(&bfree[c & 1], ((c >> 1) - 1) & 1));
-            ok = ok && __all_sync(FULL, mbar_wait(&full[s], (i / SB) & 1));
-            if (!ok) break;
-            fence_after_sync();
-            const uint64_t ad = ad0 + (uint32_t)(i % S) * (kATileBytes >> 4), bd = bd0 + (uint32_t)s * (SH::BT >> 4);
-            if (one) {
+        auto products = [&](auto log) {  // (a constant: what the loop tests stays uniform)
+            constexpr int LG = decltype(log)::value;
+            for (int i = 0; i < nst; ++i) {
+                const int s = i % SB, c = i >> LG;
+                const bool begins = i % (1 << LG) == 0;
+                if (begins && c >= 2) ok = __all_sync(FULL, mbar_wait(&bfree[c & 1], ((c >> 1) - 1) & 1));
+                ok = ok && __all_sync(FULL, mbar_wait(&full[s], (i / SB) & 1));
+                if (!ok) break;
+                fence_after_sync();
+                const uint64_t ad = ad0 + (uint32_t)(i % S) * (kATileBytes >> 4), bd = bd0 + (uint32_t)s * (SH::BT >> 4);
+                if (one) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    mma_bf16(taddr + (c & 1) * NT, ad + j * 2, bd + j * 128, kIdesc, (i % kChunk || j) ? 1u : 0u);
-                mma_commit(&empty[s]);
-                if (i % kChunk == kChunk - 1 || i == nst - 1) mma_commit(&cdone[c & 1]);
+                    for (int j = 0; j < 4; ++j)
+                        mma_bf16(taddr + (c & 1) * NT, ad + j * 2, bd + j * 128, kIdesc, (!begins || j) ? 1u : 0u);
+                    mma_commit(&empty[s]);
+                    if ((i + 1) % (1 << LG) == 0 || i == nst - 1) mma_commit(&cdone[c & 1]);
+                }
+                __syncwarp();
             }
-            __syncwarp();
+        };
+        switch (lg) {
+            case 0: products(Int<0>{}); break;
+            case 1: products(Int<1>{}); break;
+            case 2: products(Int<2>{}); break;
+            default: products(Int<kLogChunk>{});
         }
         if (!ok && one) *failed = 1;
     }
@@ -588,12 +618,45 @@ bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
     return product + bins < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
 }
 
-int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
-               cudaStream_t s) {
+// Entries of a row that an accumulator takes: up to where halving them would lessen the error.  Squared and
+// in units of 1e-16, accumulators of e entries add 0.98 e + 0.00725 e^2, and the rounding of the sums of
+// n / e of them (two of half as many up to 128 features) 1.64 n / e, or 3.1 n / e; that is within 4% of the
+// errors measured at 2,048 to 24,000 columns and 2.5 to 40% of entries, evenly spread.  (Halved where
+// that gains 4% or 10% of the rounding more than it costs.)
+static double entries_per_sum(double n, bool wide) {
+    double lo = 0, hi = kChunk * kCols;
+    for (int i = 0; i < 20; ++i) {
+        const double e = 0.5 * (lo + hi);
+        (0.49 * e + 0.00544 * e * e <= (wide ? 3.4 : 1.7) * n / e ? lo : hi) = e;
+    }
+    return lo;
+}
+
+// ... of accumulators over 512 columns or a half, a quarter, an eighth of evenly spread rows.
+static double entries_evenly(double n, int64_t K, bool wide) {
+    const double most = entries_per_sum(n, wide);
+    double e = n * kChunk * kCols / (double)K;
+    for (int k = 0; k < kLogChunk && e > most; ++k) e *= 0.5;
+    return e;
+}
+
+// The entries of a block's rows past which an accumulator's columns are halved: what evenly spread rows have
+// there, with room for their scatter (outputs do not change from block to block), or what suits the
+// accumulator if that is more.
+// 16,384 columns, 256 features: 512 columns up to 15% of entries; at 30%, 256 (error 1.44e-7 for 1.9e-7); a band of
+// 600 entries a row of 4,096 columns, one sign: 64 columns.
+static int sum_limit(int64_t M, int64_t K, int64_t nnz, bool wide) {
+    const double n = (double)nnz / (double)M, even = 1.3 * entries_evenly(n, K, wide), most = entries_per_sum(n, wide);
+    return (int)(kRows * (even > most ? even : most));
+}
+
+int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, int64_t nnz,
+               Tiles t, cudaStream_t s) {
     const int nkt = (int)col_tiles(K);
+    const int2 limit = make_int2(sum_limit(M, K, nnz, false), sum_limit(M, K, nnz, true));
     const auto kernel = !t.pos ? bin_kernel<true, false> : vals ? bin_kernel<true, true> : bin_kernel<false, true>;
     kernel<<<(unsigned)row_blocks(M), kBinThreads, sizeof(int32_t) * nkt, s>>>(rowptr, colidx, vals, (int)M, (int)K, nkt,
-                                                                               t);
+                                                                               t, limit);
     count_launches(1);
     return check_launch("tc dense regrouping");
 }

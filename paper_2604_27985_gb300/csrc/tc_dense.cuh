@@ -24,6 +24,7 @@ struct Tiles {
     uint32_t *ent;
     int32_t *tptr;
     int32_t *bad;
+    int32_t *chunk;  // per row block: log2 of the tiles of an SpMM accumulator, up to 128 features | past them << 4
     int32_t *pos;  // ent[e]'s CSR position, or null
 };
 
@@ -35,8 +36,8 @@ bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz);
 bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz);
 
 // (vals may be null where pos is not: the words then hold no values)
-int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, Tiles t,
-               cudaStream_t s);
+int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, int64_t nnz,
+               Tiles t, cudaStream_t s);
 // C = A B for N a multiple of 8 and 16-byte aligned B rows: every block of rows on the tensor
 // cores, then the marked ones (by t.bad when given, by a value that is not finite or by a wait
 // that ran out) again on the CUDA cores from p's CSR arrays.  marks: mark_count ints of scratch.

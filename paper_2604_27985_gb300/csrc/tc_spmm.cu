@@ -713,6 +713,7 @@ void plan_free(gbsp_plan *p) {
     cudaFree(p->tiles.ent);
     cudaFree(p->tiles.tptr);
     cudaFree(p->tiles.bad);
+    cudaFree(p->tiles.chunk);
     cudaFree(p->tiles.pos);
     cudaFree(p->vals_full);
     cudaFree(p->err);
@@ -878,15 +879,17 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
             dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)) == GBSP_OK &&
+            dev_alloc(&p->tiles.chunk, (size_t)dense::row_blocks(M)) == GBSP_OK &&
             dev_alloc(&p->tiles.pos, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             (fp8 || dev_alloc(&p->vals_full, (size_t)p->nnz) == GBSP_OK)) {
             if (!fp8)
                 cudaMemcpyAsync(p->vals_full, A->vals, sizeof(uint16_t) * (size_t)p->nnz, cudaMemcpyDeviceToDevice, s);
-            GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, p->vals_full, M, K, p->tiles, s));
+            GBSP_TRY(dense::launch_bin(A->rowptr, A->colidx, p->vals_full, M, K, p->nnz, p->tiles, s));
         } else {  // no room: the plan works without
             cudaFree(p->tiles.ent);
             cudaFree(p->tiles.tptr);
             cudaFree(p->tiles.bad);
+            cudaFree(p->tiles.chunk);
             cudaFree(p->tiles.pos);
             cudaFree(p->vals_full);
             p->tiles = dense::Tiles{};

@@ -266,6 +266,33 @@ def test_entries_near_2_to_the_31_stay_on_the_csr_kernels(gb):
     assert k == 2
 
 
+@pytest.mark.parametrize("band", [False, True])
+def test_dense_sums_of_one_sign(gb, band):
+    """Values and B of one sign, where everything that an accumulator cuts off adds up: 60% of 2,304 columns, and
+    rows of 600 columns in a band.  An accumulator of e entries a row is about 2.2e-9 e too small; it takes
+    at most 64 here (a full tile), 1.4e-7, beside FP32 sums of up to 36 of them (below 1e-7)."""
+    import torch
+
+    if band:
+        M, K = 12000, 4096
+        starts = np.linspace(0, K - 600, M).astype(np.int64)
+        rowptr = np.arange(M + 1, dtype=np.int32) * 600
+        colidx = (starts[:, None] + np.arange(600)).astype(np.int32).ravel()
+    else:
+        M, K = 4000, 2304
+        A = matrix(M, K, 757, 0.6, 0.6)
+        rowptr, colidx = A.rowptr, A.colidx
+    rng = np.random.default_rng(758)
+    vals, B = rng.random(colidx.size, dtype=np.float32), np.abs(gen.dense_normal(K, 64, 759))
+    plan = gb.TcPlan(dev(rowptr), dev(colidx), bf16(vals), K)
+    C, n = launches(gb, lambda: plan.execute(bf16(B)))
+    plan.check()
+    want, _ = oracle.spmm(rowptr, colidx, oracle.bf16_decode(oracle.bf16_round(vals)),
+                          oracle.bf16_decode(oracle.bf16_round(B)))
+    assert n == 2
+    assert np.linalg.norm(C.cpu().numpy() - want) <= 2.4e-7 * np.linalg.norm(want)
+
+
 @pytest.mark.parametrize("M,K,Kd,fp8", [(2048, 2048, 64, False), (2049, 2111, 192, False), (2175, 4097, 256, False),
                                         (2100, 2304, 128, True), (2303, 2049, 256, True), (2500, 2500, 384, False)])
 def test_dense_sddmm_integers_bit_exact(gb, M, K, Kd, fp8):  # (Kd = 384 in BF16: not the path)
