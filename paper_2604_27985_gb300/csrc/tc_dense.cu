@@ -578,51 +578,16 @@ bool tiles_fit(int64_t M, int64_t K, int64_t nnz) {
            row_blocks(M) * (col_tiles(K) + 1) < (1LL << 31);
 }
 
-
-// Time against time, in microseconds: a tile takes 0.30 / 0.38 / 0.46 at 64 / 128 / 256 features
-// whatever it holds, one CTA per SM, and a pair of launches 5 (measured on 2,048 to 24,000 rows and
-// columns).
-static double product_us(int64_t M, int64_t K, int64_t N, int64_t *waves) {
-    const int sms = sm_count() > 0 ? sm_count() : 1;
-    *waves = (row_blocks(M) * ((N + 255) / 256) + sms - 1) / sms;
-    return (double)(*waves * col_tiles(K)) * (N <= 64 ? 0.30 : N <= 128 ? 0.38 : 0.46) + 5.0;
+// Error of the product against 64 bits (relative 2-norm in units of 1e-8, squared) for rows of n entries, e of them
+// to an accumulator: what the accumulators lose, and the rounding of the sums of n / e of them (two of half
+// as many up to 128 features).  Within 4% of the errors measured at 2,048 to 24,000 columns and 2.5 to 40%
+// of entries, evenly spread.
+static double tile_error2(double n, double e, bool wide) {
+    return 0.98 * e + 0.00725 * e * e + (wide ? 3.1 : 1.64) * n / e;
 }
 
-// The CSR kernels split a row among 8, 4 or 2 lane groups at 64, 128 or 256 features, so short rows
-// are summed there with the smaller error: the two are level near 600 entries a row at N = 128
-// (7% of 8,192 columns: 8.2e-8 both) and near 300 at N = 256 (7% of 4,096: 7.7e-8 both).
-static bool sums_as_well(int64_t M, int64_t N, int64_t nnz) {
-    return N >= 128 && nnz >= (N < 192 ? 600 : 300) * M;
-}
-
-// The plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 / 256 features
-// where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On 16,384^2 the
-// lines cross near 6.5% / 5% / 3% of entries.  From 8% on the blocks are summed over all columns
-// on the tensor cores (error 1e-7 and more at any width), below that mostly by the CSR kernels.
-bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz) {
-    const double density = (double)nnz / ((double)M * (double)K);
-    if (M < 2048 || K < 2048 || N < 64 || N > 512 || density < 0.03) return false;
-    if (density < 0.08 && !sums_as_well(M, N, nnz)) return false;
-    int64_t waves;
-    return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
-}
-
-// For rows of even length (the split AUTO would take is the row split).  The regrouping takes 0.5 ns
-// per entry of a block of rows, the row split 13 / 24 ps per entry at 128 / 256 features: on
-// 16,384^2 the lines cross near 4.5% / 2.5% of entries, on 8,192^2 near 11% / 5%.
-bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
-    if (M < 2048 || K < 2048 || N > 512 || !sums_as_well(M, N, nnz)) return false;
-    int64_t waves;
-    const double product = product_us(M, K, N, &waves);
-    const double bins = (double)waves * 0.5e-3 * (double)nnz / (double)row_blocks(M);
-    return product + bins < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
-}
-
-// Entries of a row that an accumulator takes: up to where halving them would lessen the error.  Squared and
-// in units of 1e-16, accumulators of e entries add 0.98 e + 0.00725 e^2, and the rounding of the sums of
-// n / e of them (two of half as many up to 128 features) 1.64 n / e, or 3.1 n / e; that is within 4% of the
-// errors measured at 2,048 to 24,000 columns and 2.5 to 40% of entries, evenly spread.  (Halved where
-// that gains 4% or 10% of the rounding more than it costs.)
+// Entries of a row that an accumulator takes: up to where halving them would lessen that error (by 4% or 10% of
+// the rounding more than it costs).
 static double entries_per_sum(double n, bool wide) {
     double lo = 0, hi = kChunk * kCols;
     for (int i = 0; i < 20; ++i) {
@@ -648,6 +613,52 @@ static double entries_evenly(double n, int64_t K, bool wide) {
 static int sum_limit(int64_t M, int64_t K, int64_t nnz, bool wide) {
     const double n = (double)nnz / (double)M, even = 1.3 * entries_evenly(n, K, wide), most = entries_per_sum(n, wide);
     return (int)(kRows * (even > most ? even : most));
+}
+
+// Time against time, in microseconds: a tile takes 0.30 / 0.38 / 0.46 at 64 / 128 / 256 features
+// whatever it holds, one CTA per SM, and a pair of launches 5 (measured on 2,048 to 24,000 rows and
+// columns).
+static double product_us(int64_t M, int64_t K, int64_t N, int64_t *waves) {
+    const int sms = sm_count() > 0 ? sm_count() : 1;
+    *waves = (row_blocks(M) * ((N + 255) / 256) + sms - 1) / sms;
+    return (double)(*waves * col_tiles(K)) * (N <= 64 ? 0.30 : N <= 128 ? 0.38 : 0.46) + 5.0;
+}
+
+// Whether the sums are as exact as the CSR kernels', which split a row among 8, 4 or 2 lane groups at 64,
+// 128 or 256 features: their squared error is 0.116 / 0.207 / 0.37 n at 128 / 256 / more features (within 3%
+// of the measured ones).  At 128 features that is from about 660 entries a row on (660 of 2,049 columns: 8.6e-8
+// both; 600 of 5,000 at 12%: 8.0e-8 against 8.3e-8), at 256 from about 360 (12,288 columns at 4%: 9.5e-8 against
+// 1.0e-7; 3,000 at 11%: 8.5e-8 against 8.2e-8), but not on so few entries per tile that the rounding of the
+// sums outweighs (16,384 columns at 2.5%, 256 features: 9.6e-8 against 9.2e-8).
+// With values and B of one sign the CSR kernels' rounding does not add up and the accumulators' loss
+// does: on the same sizes 0.4 to 0.95 of the CSR kernels' error from 129 features on, 0.7 to 1.3 at 128.
+static bool sums_as_well(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    if (N < 128) return false;
+    const double n = (double)nnz / (double)M;
+    return tile_error2(n, entries_evenly(n, K, N > 128), N > 128) <= (N <= 128 ? 0.116 : N <= 256 ? 0.207 : 0.37) * n;
+}
+
+// The plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 / 256 features
+// where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On 16,384^2 the
+// lines cross near 6.5% / 5% / 3% of entries.  From 8% on the blocks are summed over all columns
+// on the tensor cores (error 1e-7 and more at any width), below that mostly by the CSR kernels.
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    const double density = (double)nnz / ((double)M * (double)K);
+    if (M < 2048 || K < 2048 || N < 64 || N > 512 || density < 0.03) return false;
+    if (density < 0.08 && !sums_as_well(M, K, N, nnz)) return false;
+    int64_t waves;
+    return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+}
+
+// For rows of even length (the split AUTO would take is the row split).  The regrouping takes 0.5 ns
+// per entry of a block of rows, the row split 13 / 24 ps per entry at 128 / 256 features: on
+// 16,384^2 the lines cross near 4.5% / 2.5% of entries, on 8,192^2 near 11% / 5%.
+bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    if (M < 2048 || K < 2048 || N > 512 || !sums_as_well(M, K, N, nnz)) return false;
+    int64_t waves;
+    const double product = product_us(M, K, N, &waves);
+    const double bins = (double)waves * 0.5e-3 * (double)nnz / (double)row_blocks(M);
+    return product + bins < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
 }
 
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, int64_t nnz,
