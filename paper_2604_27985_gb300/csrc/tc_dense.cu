@@ -640,12 +640,16 @@ static bool sums_as_well(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 
 // The plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 / 256 features
 // where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On 16,384^2 the
-// lines cross near 6.5% / 5% / 3% of entries.  From 8% on the blocks are summed over all columns
-// on the tensor cores (error 1e-7 and more at any width), below that mostly by the CSR kernels.
-bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz) {
-    const double density = (double)nnz / ((double)M * (double)K);
-    if (M < 2048 || K < 2048 || N < 64 || N > 512 || density < 0.03) return false;
-    if (density < 0.08 && !sums_as_well(M, K, N, nnz)) return false;
+// lines cross near 6.5% / 5% / 3% of entries.
+// Its blocks' MMAs run one accumulator over all of a row's entries in blocks, the share s of them, and so lose
+// about s^2 K / 512 times what whole tiles do: at 512 the errors are level (2,048 columns, half in
+// blocks: 1.00 at 2.5% of entries, 0.79 at 10%), above that whole tiles have the smaller one (0.13 of it
+// on 16,384 columns at 10%), below it only where their sums are as exact as the CSR kernels', which
+// then have most of the entries (8% of 3,072 columns, a fifth in blocks: 6.2e-8 against 7.3e-8 at 64 features).
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz) {
+    if (M < 2048 || K < 2048 || N < 64 || N > 512 || (double)nnz < 0.03 * (double)M * (double)K) return false;
+    const double share = (double)dense_nnz / (double)nnz;
+    if ((double)K * share * share < kChunk * kCols && !sums_as_well(M, K, N, nnz)) return false;
     int64_t waves;
     return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
 }

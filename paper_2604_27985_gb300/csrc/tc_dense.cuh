@@ -31,7 +31,8 @@ struct Tiles {
 // Whether the regrouping is possible for these sizes (entry positions are 32-bit and run up to 2,048 past
 // the last entry), and whether it is worth it.
 bool tiles_fit(int64_t M, int64_t K, int64_t nnz);
-bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz);
+// (dense_nnz: the entries that a plan's 16 x 8 blocks would hold)
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz);
 // ... also where the regrouping is part of every call, against the CSR kernels.
 bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz);
 

@@ -875,7 +875,8 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
     if (by_default && dense::tiles_fit(M, K, p->nnz) &&
-        (dense::spmm_pays(M, K, 256, p->nnz) || dense::sddmm_pays(M, K, 256, p->nnz, fp8))) {
+        (dense::spmm_pays(M, K, 256, p->nnz, p->dense_nnz) || dense::spmm_pays(M, K, 512, p->nnz, p->dense_nnz) ||
+         dense::sddmm_pays(M, K, 256, p->nnz, fp8))) {
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
             dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)) == GBSP_OK &&
@@ -992,7 +993,7 @@ GBSP_EXPORT int gbsp_plan_execute(const gbsp_plan *p, const gbsp_dense *B, gbsp_
     // (whole tiles store groups of 8 columns and copy B in 16-byte pieces; a plan without dense windows takes
     // any other B on the CSR kernels below)
     const bool whole = !fp8 && p->tiles.ent && N % 8 == 0 && B->ld % 8 == 0 && aligned16(B->data) &&
-                       dense::spmm_pays(p->M, p->K, N, p->nnz);
+                       dense::spmm_pays(p->M, p->K, N, p->nnz, p->dense_nnz);
     if (whole && injected_fault() == 2)
         return fail(GBSP_ERR_CUDA, "plan execute: injected launch failure (GBSP_FAULT=launch)");
     void *marks = nullptr;

@@ -287,6 +287,29 @@ def test_dense_without_a_plan_is_as_exact_as_the_row_split(gb, M, K, N, density,
     assert error(C) <= 1.04 * error(gb.spmm(rp, ci, v, b, variant="rowsplit"))
 
 
+@pytest.mark.parametrize("M,K,N,density,whole", [(12000, 3072, 64, 0.08, False), (12000, 6144, 128, 0.08, False),
+                                                 (12000, 3072, 64, 0.12, True), (9000, 3072, 264, 0.08, True)])
+def test_dense_plan_is_as_exact_as_its_blocks(gb, M, K, N, density, whole):
+    """A plan takes whole tiles only where their error against 64 bits is that of its blocks and CSR residual
+    (here a fifth of the entries in blocks at 8%, three quarters at 12%) or less."""
+    import torch
+
+    g = torch.Generator("cuda").manual_seed(745)
+    n = round(density * K)
+    at = torch.rand(M, K, device="cuda", generator=g).topk(n, 1).indices.sort(1).values
+    rp, ci = torch.arange(M + 1, dtype=torch.int32, device="cuda") * n, at.int().reshape(-1).contiguous()
+    v = (torch.rand(M * n, device="cuda", generator=g) * 2 - 1).bfloat16()
+    b = torch.randn(K, N, device="cuda", generator=g).bfloat16()
+    plan, blocks = gb.TcPlan(rp, ci, v, K), gb.TcPlan(rp, ci, v, K, threshold=14)
+    C, other = plan.execute(b), blocks.execute(b)
+    plan.check()
+    blocks.check()
+    want = torch.sparse_csr_tensor(rp, ci, v.double(), size=(M, K)) @ b.double()
+    error = lambda x: float((x.double() - want).norm() / want.norm())
+    assert torch.equal(C, other) != whole
+    assert error(C) <= 1.04 * error(other)
+
+
 @pytest.mark.parametrize("band", [False, True])
 def test_dense_sums_of_one_sign(gb, band):
     """Values and B of one sign, where everything that an accumulator cuts off adds up: 60% of 2,304 columns, and
