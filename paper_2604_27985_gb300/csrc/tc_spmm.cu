@@ -1103,11 +1103,13 @@ GBSP_EXPORT int gbsp_plan_sddmm(const gbsp_plan *p, const float *svals, const gb
     // the tiles pay when a dense block holds enough stored entries to outweigh gathering all
     // its 8 Y rows (measured crossover between 16 and 27 per block on 16,384^2 at 90%, Kd = 256)
     if (tiles < 0) tiles = p->nwin_tc > 0 && p->dense_nnz >= 24 * p->nblocks;
-    // whole 128 x 64 tiles (tc_dense_sddmm.cu) where the sums were the tensor cores' already (from
-    // Kd = 64 on its short parts are the more exact ones) or E4M3's, which are as exact as the CSR
-    // kernels'
-    const bool whole = by_default && p->tiles.pos && (tiles || (fp8 && Kd <= 256)) &&
-                       dense::sddmm_pays(p->M, p->K, Kd, p->nnz, fp8);
+    // Whole 128 x 64 tiles (tc_dense_sddmm.cu) where they are as exact: E4M3's sums are (their value and
+    // scales are rounded once); BF16's where a seventh of the entries would be in the blocks, whose one
+    // accumulator over Kd loses more than the whole tiles' four.  Errors of the CSR kernel / whole tiles /
+    // block entries at Kd = 64, 128, 256: 4.7 / 5.05 / 7.0, 5.5 / 6.15 / 11.9, 6.1 / 8.1 / 23 (e-8), level with 13%,
+    // 7% and 6% of the entries in blocks.
+    const bool exact = fp8 ? tiles || Kd <= 256 : tiles && 7 * p->dense_nnz >= p->nnz;
+    const bool whole = by_default && p->tiles.pos && exact && dense::sddmm_pays(p->M, p->K, Kd, p->nnz, fp8);
     if (tiles && p->nwin_tc > 0 && ((Kd * es) % 128 || kb < 1 || kb > 8))
         return fail(GBSP_ERR_UNSUPPORTED, "plan sddmm: tensor-core tiles need Kd a multiple of %d and at most %d",
                     128 / es, 1024 / es);

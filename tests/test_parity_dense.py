@@ -360,6 +360,31 @@ def test_dense_sddmm_integers_bit_exact(gb, M, K, Kd, fp8):  # (Kd = 384 in BF16
     assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
 
 
+@pytest.mark.parametrize("blocks,whole", [(1000, False), (4000, True)])
+def test_dense_sddmm_is_as_exact_as_the_blocks(gb, blocks, whole):
+    """5% of entries anywhere and full 16 x 8 blocks: whole tiles are the more exact ones only where the blocks
+    hold a fair share (a seventh) of the entries, else the residual's CSR kernel has most of them."""
+    import torch
+
+    M, K, Kd = 8192, 4096, 256
+    g = torch.Generator("cuda").manual_seed(775)
+    mask = torch.rand(M, K, device="cuda", generator=g) < 0.05
+    at = torch.randperm(M // 16 * (K // 8), device="cuda", generator=g)[:blocks]
+    mask.view(M // 16, 16, K // 8, 8)[at // (K // 8), :, at % (K // 8), :] = True
+    row, col = mask.nonzero(as_tuple=True)
+    rp = torch.zeros(M + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = mask.sum(1).cumsum(0).int()
+    sv = torch.rand(row.numel(), device="cuda", generator=g) * 2 - 1
+    x, y = (torch.randn(n, Kd, device="cuda", generator=g).bfloat16() for n in (M, K))
+    plan = gb.TcPlan(rp, col.int(), sv.bfloat16(), K)
+    out, n = launches(gb, lambda: plan.sddmm(sv, x, y))
+    plan.check()
+    assert n == (1 if whole else 2)
+    want = (x.double()[row] * y.double()[col]).sum(1) * sv.double()
+    error = lambda o: float((o.double() - want).norm() / want.norm())
+    assert error(out) <= error(plan.sddmm(sv, x, y, tiles=1))
+
+
 def test_dense_sddmm_random_scales_and_infinities(gb):
     """E4M3 row scales on an E4M3 plan, padded leading dimensions; an infinity or NaN in an X or Y
     row reaches only that row's entries."""
