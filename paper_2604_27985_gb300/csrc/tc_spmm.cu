@@ -874,8 +874,10 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     }
     // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
+    // (an E4M3 plan's SpMM does not take them)
     if (by_default && dense::tiles_fit(M, K, p->nnz) &&
-        (dense::spmm_pays(M, K, 256, p->nnz, p->dense_nnz) || dense::spmm_pays(M, K, 512, p->nnz, p->dense_nnz) ||
+        ((!fp8 && (dense::spmm_pays(M, K, 256, p->nnz, p->dense_nnz) ||
+                   dense::spmm_pays(M, K, 512, p->nnz, p->dense_nnz))) ||
          dense::sddmm_pays(M, K, 256, p->nnz, fp8))) {
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&

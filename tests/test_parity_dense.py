@@ -360,6 +360,24 @@ def test_dense_sddmm_integers_bit_exact(gb, M, K, Kd, fp8):  # (Kd = 384 in BF16
     assert np.array_equal(out.cpu().numpy().astype(np.float64), want)
 
 
+def test_e4m3_plan_keeps_no_tiles_for_its_spmm(gb):
+    """Where only a BF16 SpMM would take whole tiles (3.1% of entries here), an E4M3 plan holds its copies of the
+    pattern, the positions and the values, 13 bytes per entry, and not the tiles' 8 beside them."""
+    import torch
+
+    M, K, n = 19456, 16384, 514
+    ci = (torch.arange(n, device="cuda") * 31 + torch.arange(M, device="cuda")[:, None] * 7 % 31).int().reshape(-1)
+    rp = torch.arange(M + 1, dtype=torch.int32, device="cuda") * n
+    v = torch.ones(M * n, device="cuda").to(torch.float8_e4m3fn).view(torch.uint8)
+    s = torch.ones(M, device="cuda")
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    plan = gb.TcPlan(rp, ci, v, K, row_scale=s)
+    used = before - torch.cuda.mem_get_info()[0]
+    assert plan.info()["dense_windows"] == 0
+    assert used <= 15 * M * n
+
+
 @pytest.mark.parametrize("blocks,whole", [(1000, False), (4000, True)])
 def test_dense_sddmm_is_as_exact_as_the_blocks(gb, blocks, whole):
     """5% of entries anywhere and full 16 x 8 blocks: whole tiles are the more exact ones only where the blocks
