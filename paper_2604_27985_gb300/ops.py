@@ -7,7 +7,6 @@ SpMM / SDDMM happens here; PyTorch only owns the memory and the stream.
 from __future__ import annotations
 
 import ctypes
-import functools
 import struct
 
 import torch
@@ -91,9 +90,8 @@ def _dense_bytes(t, scale=None) -> bytes:
     return _DENSE.pack(_ptr(t) or 0, shape[0], shape[1], _ld(t), _ptr(scale) or 0, _dtype(t))
 
 
-@functools.lru_cache(maxsize=256)
 def _opts_bytes(variant, validate, unroll, ctas_per_sm, vecs) -> bytes:
-    return _OPTS.pack(VARIANTS[variant] if isinstance(variant, str) else int(variant), int(bool(validate)),
+    return _OPTS.pack(VARIANTS[variant] if isinstance(variant, str) else int(variant), bool(validate),
                       int(unroll), int(ctas_per_sm), int(vecs))
 
 

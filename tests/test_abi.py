@@ -92,6 +92,20 @@ def test_argument_errors_return_without_launching(gb):
     assert lib.gbsp_get_last_error() == -1
 
 
+def test_options_are_read_on_every_call(gb):
+    """Option values that are arrays are taken as numbers, at their value of the moment."""
+    import struct
+
+    import numpy as np
+
+    from paper_2604_27985_gb300 import ops
+
+    vecs = np.array(2)
+    for v in (2, 4):
+        vecs[...] = v
+        assert ops._opts_bytes("rowsplit", np.array(False), 0, 0, vecs) == struct.pack("5i", 1, 0, 0, 0, v)
+
+
 def _run_with_fault(fault, code):
     import subprocess
     import sys
