@@ -89,7 +89,7 @@ int scratch_alloc(void **ptr, size_t bytes, cudaStream_t s) {
                 cudaGetLastError();
                 return fail(GBSP_ERR_OOM, "workspace pool creation failed");
             }
-            uint64_t keep = 1ull << 30;  // freed workspace kept for the next call; past it, given back
+            uint64_t keep = kPoolKeep;
             cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
         }
     }

@@ -14,6 +14,7 @@ namespace gbsp {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+constexpr uint64_t kPoolKeep = 1ull << 30;  // bytes of freed workspace kept for the next call; past it, given back
 // Records a failure for gbsp_get_last_error / gbsp_last_error_message and returns status.
 int fail(int status, const char *fmt, ...);
 // Clears the per-thread error record and returns GBSP_OK.

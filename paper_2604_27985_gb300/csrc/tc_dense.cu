@@ -662,7 +662,7 @@ bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz) {
     int64_t waves;
     const double product = product_us(M, K, N, &waves);
     const double bins = (double)waves * 0.5e-3 * (double)nnz / (double)row_blocks(M);
-    return product + bins < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
+    return product + bins + scratch_us(4 * nnz) < 0.85e-6 * (double)nnz * (2.3 + 0.085 * (double)N);
 }
 
 int launch_bin(const int32_t *rowptr, const int32_t *colidx, const uint16_t *vals, int64_t M, int64_t K, int64_t nnz,

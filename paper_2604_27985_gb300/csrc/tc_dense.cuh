@@ -28,6 +28,13 @@ struct Tiles {
     int32_t *pos;  // ent[e]'s CSR position, or null
 };
 
+// Microseconds that a call's scratch costs beside its kernels: what the pool does not keep is mapped anew after
+// every synchronisation (1.2 GB 0.4 ms, 1.9 GB 1.7, 3.4 GB 4.3, 4.0 GB 5.3; a little less is counted, since not
+// every call is followed by one).
+inline double scratch_us(int64_t bytes) {
+    return bytes > (int64_t)kPoolKeep ? 1.6e-6 * (double)(bytes - (int64_t)kPoolKeep) : 0.0;
+}
+
 // Whether the regrouping is possible for these sizes (entry positions are 32-bit and run up to 2,048 past
 // the last entry), and whether it is worth it.
 bool tiles_fit(int64_t M, int64_t K, int64_t nnz);

@@ -429,13 +429,16 @@ bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8) {
 // time).  E4M3 only: at Kd <= 256 its error is below the CSR kernel's (3.0e-8 against 4.55e-8 on
 // 16,384^2 at 90%, Kd = 256), BF16's four steps per part have the larger one
 // (8.0e-8 against 6.1e-8).  The E4M3 CSR kernel is bound by its conversions: 16 / 30 ps per entry at
-// Kd = 128 / 256.
+// Kd = 128 / 256.  Where the scratch passes the pool's limit (from 134 million entries on) a tile was measured at
+// 1.6 to 2.2 ns an entry: 300 million, calls waited for, Kd = 128 7.7 ms against 4.3 for the row split, Kd = 256
+// 7.7 against 8.4; 138 million 2.3 against 2.1 and 2.4 against 3.9.
 bool sddmm_pays_unplanned(int64_t M, int64_t K, int64_t Kd, int64_t nnz) {
     if (M < 2048 || K < 2048 || Kd > 256 || Kd < 128 || (double)nnz < 0.03 * (double)M * (double)K) return false;
     const int64_t sms = sm_count() > 0 ? sm_count() : 1, nb = row_blocks(M);
-    const double tile = 0.95 * (double)(nb * col_tiles(K)) / (double)sms;
+    const double held = (double)nnz / (double)(nb * col_tiles(K)), remap = scratch_us(8 * nnz);
+    const double tile = (remap > 0 && held > 560 ? 1.7e-3 * held : 0.95) * (double)(nb * col_tiles(K)) / (double)sms;
     const double bins = (double)((nb + sms - 1) / sms) * 0.6e-3 * (double)nnz / (double)nb;
-    return tile + bins + 12.0 < 0.85e-6 * (double)nnz * (2.5 + 0.105 * (double)Kd);
+    return tile + bins + 12.0 + remap < 0.85e-6 * (double)nnz * (2.5 + 0.105 * (double)Kd);
 }
 
 int launch_sddmm(const SddmmProblem &p, Tiles t, int *err, int withhold, cudaStream_t s) {

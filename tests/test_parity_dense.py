@@ -488,3 +488,22 @@ def test_dense_sddmm_scales_and_value_round_once(gb, Kd):
     want = dots * svals * np.repeat(f64(sx), np.diff(A.rowptr)) * f64(sy)[A.colidx]
     assert n == 4
     assert np.all(np.abs(f64(out) - want) <= 2.0**-24 * (1 + 1e-6) * np.abs(want))
+
+
+def test_dense_sddmm_scratch_past_the_pool_is_counted(gb):
+    """300 million entries need 2.4 GB of scratch, most of which the pool gives back after each call: at Kd = 128
+    the row split is then the faster one (the statistics and one launch)."""
+    import torch
+
+    M, K, n = 65536, 49152, 4577
+    ci = (torch.arange(n, device="cuda", dtype=torch.int32) * 10 +
+          (torch.arange(M, device="cuda", dtype=torch.int32) % 10)[:, None]).reshape(-1)
+    rp = torch.arange(M + 1, dtype=torch.int32, device="cuda") * n
+    X, Y = gen.dense_int(M, 128, 799, -4, 4), gen.dense_int(K, 128, 800, -4, 4)
+    one = lambda k: torch.ones(k, device="cuda")
+    out, k = launches(gb, lambda: gb.sddmm(rp, ci, one(M * n), dev(oracle.e4m3_round(X)), dev(oracle.e4m3_round(Y)),
+                                           x_scale=one(M), y_scale=one(K)))
+    assert k == 2
+    for r in (0, 777, M - 1):
+        cols = ci[r * n:(r + 1) * n].cpu().numpy()
+        assert np.array_equal(out[r * n:(r + 1) * n].cpu().numpy(), Y[cols] @ X[r])
