@@ -721,6 +721,11 @@ void plan_free(gbsp_plan *p) {
 }
 
 
+// Whether an SDDMM uses the blocks by default: they pay when a dense block holds enough stored
+// entries to outweigh gathering all its 8 Y rows (measured crossover between 16 and 27 per block
+// on 16,384^2 at 90%, Kd = 256).
+bool takes_tiles(const gbsp_plan *p) { return p->nwin_tc > 0 && p->dense_nnz >= 24 * p->nblocks; }
+
 template <int NT, bool FP8>
 int launch_tc(const CUtensorMap &map, const TcArgs &args, int nwin, int ngroups, cudaStream_t s) {
     using SH = TcShape<NT, FP8>;
@@ -874,11 +879,12 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     }
     // A caller who sets neither the threshold nor the residual's kernel leaves the arithmetic to
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
-    // (an E4M3 plan's SpMM does not take them)
+    // (an E4M3 plan's SpMM does not take them, its SDDMM past Kd = 256 where the tiles do)
     if (by_default && dense::tiles_fit(M, K, p->nnz) &&
         ((!fp8 && (dense::spmm_pays(M, K, 256, p->nnz, p->dense_nnz) ||
                    dense::spmm_pays(M, K, 512, p->nnz, p->dense_nnz))) ||
-         dense::sddmm_pays(M, K, 256, p->nnz, fp8))) {
+         dense::sddmm_pays(M, K, 256, p->nnz, fp8) ||
+         (fp8 && takes_tiles(p) && dense::sddmm_pays(M, K, dense::sddmm_max_kd(fp8), p->nnz, fp8)))) {
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
             dev_alloc(&p->tiles.bad, (size_t)dense::row_blocks(M)) == GBSP_OK &&
@@ -1102,9 +1108,7 @@ GBSP_EXPORT int gbsp_plan_sddmm(const gbsp_plan *p, const float *svals, const gb
                                     "Y, Kd <= 512", V);
     const int kb = (int)(Kd * es / 128);
     const bool by_default = tiles < 0;
-    // the tiles pay when a dense block holds enough stored entries to outweigh gathering all
-    // its 8 Y rows (measured crossover between 16 and 27 per block on 16,384^2 at 90%, Kd = 256)
-    if (tiles < 0) tiles = p->nwin_tc > 0 && p->dense_nnz >= 24 * p->nblocks;
+    if (tiles < 0) tiles = takes_tiles(p);
     // Whole 128 x 64 tiles (tc_dense_sddmm.cu) where they are as exact: E4M3's sums are (their value and
     // scales are rounded once); BF16's where a seventh of the entries would be in the blocks, whose one
     // accumulator over Kd loses more than the whole tiles' four.  Errors of the CSR kernel / whole tiles /

@@ -378,6 +378,29 @@ def test_e4m3_plan_keeps_no_tiles_for_its_spmm(gb):
     assert used <= 15 * M * n
 
 
+def test_e4m3_plan_wide_sddmm_takes_whole_tiles(gb):
+    """4.4% of entries, most in full 16 x 8 blocks: at Kd = 512 whole tiles pay, at 256 they do not."""
+    import torch
+
+    M, K = 4096, 4096
+    g = torch.Generator("cuda").manual_seed(777)
+    at = torch.randperm(M // 16 * (K // 8), device="cuda", generator=g)[:5500]
+    mask = torch.rand(M // 16, 16, K // 8, 8, device="cuda", generator=g) < 0.002
+    mask[at // (K // 8), :, at % (K // 8), :] = True
+    row, col = mask.view(M, K).nonzero(as_tuple=True)
+    rp = torch.zeros(M + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = mask.view(M, K).sum(1).cumsum(0).int()
+    v = torch.ones(row.numel(), device="cuda")
+    plan = gb.TcPlan(rp, col.int(), v.to(torch.float8_e4m3fn).view(torch.uint8), K, row_scale=torch.ones(M, device="cuda"))
+    one = torch.ones(K, device="cuda")
+    for Kd, whole in ((256, False), (512, True)):
+        X, Y = gen.dense_int(M, Kd, 778, -4, 4), gen.dense_int(K, Kd, 779, -4, 4)
+        out, n = launches(gb, lambda: plan.sddmm(v, dev(oracle.e4m3_round(X)), dev(oracle.e4m3_round(Y)), x_scale=one, y_scale=one))
+        plan.check()
+        assert (n == 1) == whole
+        assert torch.equal(out.double(), (dev(X).double()[row] * dev(Y).double()[col]).sum(1))
+
+
 @pytest.mark.parametrize("blocks,whole", [(1000, False), (4000, True)])
 def test_dense_sddmm_is_as_exact_as_the_blocks(gb, blocks, whole):
     """5% of entries anywhere and full 16 x 8 blocks: whole tiles are the more exact ones only where the blocks
