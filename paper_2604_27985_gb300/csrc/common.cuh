@@ -200,6 +200,26 @@ __device__ __forceinline__ void unit_decode(const Unit<LB> &u, float (&o)[LB / (
     }
 }
 
+// One element in a 32-bit register (16-bit ones would be packed in pairs and taken apart again), and its value.
+__device__ __forceinline__ uint32_t ld_word(const float *p) { return __float_as_uint(__ldg(p)); }
+__device__ __forceinline__ uint32_t ld_word(const uint16_t *p) {
+    uint32_t w;
+    asm("ld.global.nc.u16 %0, [%1];" : "=r"(w) : "l"(p));
+    return w;
+}
+__device__ __forceinline__ uint32_t ld_word(const uint8_t *p) {
+    uint32_t w;
+    asm("ld.global.nc.u8 %0, [%1];" : "=r"(w) : "l"(p));
+    return w;
+}
+template <class EL>
+__device__ __forceinline__ float word_value(uint32_t w) {
+    if constexpr (sizeof(typename EL::stored) == 4)
+        return __uint_as_float(w);
+    else
+        return EL::value((typename EL::stored)w);
+}
+
 // Streaming (read-once) loads: indices and values are touched once, so keep them from
 // displacing the gathered dense rows in L1 / L2.
 __device__ __forceinline__ int ld_stream(const int32_t *p) { return __ldcs(p); }

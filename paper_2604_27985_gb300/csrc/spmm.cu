@@ -5,42 +5,69 @@ namespace gbsp {
 
 // Units per lane: what covers the row, at most 8 (FP32 sums of at most 16 elements a lane).
 template <class EL, int LB>
-int launch_scalar(const SpmmProblem &P, cudaStream_t s) {
+int launch_units(const SpmmProblem &P, cudaStream_t s) {
     using namespace spmm_detail;
-    constexpr int UE = LB / (int)sizeof(typename EL::stored), TMAX = UE >= 8 ? 2 : UE >= 4 ? 4 : 8;
+    // (single elements: FP32 up to 64, the others up to 64 and past 128)
+    constexpr int ES = (int)sizeof(typename EL::stored), UE = LB / ES;
+    constexpr int TMAX = UE >= 8 || (UE == 1 && ES == 4) ? 2 : UE >= 4 ? 4 : 8;
     const int units = P.N / UE;
     const dim3 grid((P.M + 7) / 8);
     if (units <= 32)
         spmm_unit_kernel<EL, LB, 1><<<grid, 256, 0, s>>>(P);
     else if (units <= 64 || TMAX == 2)
         spmm_unit_kernel<EL, LB, 2><<<grid, 256, 0, s>>>(P);
+    else if constexpr (UE == 1)
+        spmm_unit_kernel<EL, LB, TMAX><<<grid, 256, 0, s>>>(P);
     else if (units <= 128 || TMAX == 4)
         spmm_unit_kernel<EL, LB, TMAX < 4 ? TMAX : 4><<<grid, 256, 0, s>>>(P);
     else
         spmm_unit_kernel<EL, LB, TMAX><<<grid, 256, 0, s>>>(P);
     count_launches(1);
+    return check_launch("spmm units");
+}
+
+template <class EL, int U, int T>
+int launch_elements(const SpmmProblem &P, cudaStream_t s) {
+    spmm_detail::spmm_scalar_kernel<EL, U, T><<<dim3((P.M + 7) / 8), 256, 0, s>>>(P);
+    count_launches(1);
     return check_launch("spmm scalar");
+}
+
+// The unvectorised kernels, by what the rows' alignment allows (lb bytes a load) and what was measured on 30,011
+// x 41,017 (20 and 205 entries a row, even and Zipf), 4,000 x 41,017 (1,500), 200,000 x 3,000 (100), 3,000 x 3,000
+// (200) and 20,000 x 250,000 (60, clustered), times of the first of two over the second:
+// - rows averaging under 16 entries (or not said): one entry at a time.  200,000 x 3,000, 6 entries a row,
+//   N = 101: 85 us against 117 for the units.
+// - wide loads that leave half of the lanes without one are halved: E4M3 N = 24 to 120 from 8 bytes 1.4 to 2.8
+//   times as fast; the others level or better.
+// - 65 to 96 single elements: three columns a lane, four entries in flight, 0.43 to 1.04 of one at a time's time and
+//   0.67 to 0.88 of the units' (four columns).
+// - more of them: FP32 four columns and entries, 0.81 to 1.05 of the units' time (0.48 to 1.01 of one at a time's);
+//   E4M3 up to 128 the same, 0.89 to 1.02.  BF16 up to 128 one at a time: 0.74 to 0.99 of the units' time
+//   on even rows (1.12 on the 3,000, 1.6 on the Zipf ones), 0.82 to 0.99 of four in flight's (1.25).  E4M3 and
+//   BF16 past that the units: one at a time takes 0.79 to 1.22 of their time (Zipf 1.7).
+template <class EL>
+int launch_unvectorised(const SpmmProblem &P, cudaStream_t s) {
+    constexpr int ES = (int)sizeof(typename EL::stored);
+    if (P.nnz < 16LL * P.M) return launch_elements<EL, 1, 4>(P, s);
+    int lb = unit_bytes(P.B, P.ldb, P.N, ES);
+    while (lb > ES && P.N * ES < 16 * lb) lb /= 2;
+    if (lb == ES && P.N > 64) {
+        if (P.N <= 96) return launch_elements<EL, 4, 3>(P, s);
+        if (ES == 2 && P.N <= 128) return launch_elements<EL, 1, 4>(P, s);
+        if constexpr (ES != 2)
+            if (ES == 4 || P.N <= 128) return launch_elements<EL, 4, 4>(P, s);
+    }
+    if constexpr (ES <= 1)
+        if (lb == 1) return launch_units<EL, 1>(P, s);
+    if constexpr (ES <= 2)
+        if (lb == 2) return launch_units<EL, 2>(P, s);
+    return lb == 4 ? launch_units<EL, 4>(P, s) : launch_units<EL, 8>(P, s);
 }
 
 template <class EL>
 int launch_spmm_typed(const SpmmProblem &P, int variant, int vecs, int unroll, int ctas_per_sm, cudaStream_t s) {
-    if (variant == GBSP_VARIANT_SCALAR) {
-        // rows averaging under 16 entries (or not said): 200,000 x 3,000, 6 entries a row, N = 101: 85 us
-        // against 117 for the units; and 65 to 128 single BF16 elements a row: 287 us against 299 on 30,011 x
-        // 41,017, N = 101
-        constexpr int ES = (int)sizeof(typename EL::stored);
-        const int lb = unit_bytes(P.B, P.ldb, P.N, ES);
-        if (P.nnz < 16LL * P.M || (ES == 2 && lb == 2 && P.N > 64 && P.N <= 128)) {
-            spmm_detail::spmm_scalar_kernel<EL><<<dim3((P.M + 7) / 8, 1), 256, 0, s>>>(P);
-            count_launches(1);
-            return check_launch("spmm scalar");
-        }
-        if constexpr (ES <= 1)
-            if (lb == 1) return launch_scalar<EL, 1>(P, s);
-        if constexpr (ES <= 2)
-            if (lb == 2) return launch_scalar<EL, 2>(P, s);
-        return lb == 4 ? launch_scalar<EL, 4>(P, s) : launch_scalar<EL, 8>(P, s);
-    }
+    if (variant == GBSP_VARIANT_SCALAR) return launch_unvectorised<EL>(P, s);
     if (variant == GBSP_VARIANT_MERGE) return launch_spmm_algo<EL, GBSP_VARIANT_MERGE>(P, vecs, unroll, ctas_per_sm, s);
     if (variant == GBSP_VARIANT_ROWGROUP)
         return launch_spmm_algo<EL, GBSP_VARIANT_ROWGROUP>(P, vecs, unroll, ctas_per_sm, s);

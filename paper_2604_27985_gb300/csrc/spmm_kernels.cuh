@@ -428,18 +428,25 @@ __global__ void __launch_bounds__(256) spmm_unit_kernel(const SpmmProblem P) {
     }
 }
 
-// ... for rows of a few entries, which the units' registers (fewer warps per SM) do not help: one warp per row, lane l owns columns
-// l, l + 32, l + 64, l + 96 of a 128-column pass.
-template <class EL>
+// ... element by element, lane l owns columns l, l + 32, ... of a pass of T x 32, U entries' loads in flight and
+// the columns past the row's end predicated.  U = 1: rows of a few entries, where the registers of
+// more (fewer warps per SM) do not help.  U = 4, 40 to 62 registers where the units take 76 to 80, so that
+// rows from a B close at hand (200,000 x 3,000, 100 entries a row: FP32 N = 65 / 127 624 / 740 us at U = 1, 867 /
+// 880 with the units, 587 / 718 so) keep their warps and long rows (30,011 x 41,017, 205 entries a row,
+// Zipf: 1029 / 1404, 731 / 730, 607 / 688) their loads.
+template <class EL, int U, int T>
 __global__ void __launch_bounds__(256) spmm_scalar_kernel(const SpmmProblem P) {
+    using ST = typename EL::stored;
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= P.M) return;
     const int64_t p0 = __ldg(P.rowptr + row), p1 = __ldg(P.rowptr + row + 1);
-    const typename EL::stored *B = static_cast<const typename EL::stored *>(P.B);
+    const ST *B = static_cast<const ST *>(P.B);
     const float sc = row_scale<EL>(P, row);
-    for (int c0 = blockIdx.y * 128; c0 < P.N; c0 += gridDim.y * 128) {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int c0 = lane; c0 - lane < P.N; c0 += 32 * T) {
+        float acc[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t) acc[t] = 0.f;
         for (int64_t base = p0; base < p1; base += 32) {
             int c = 0;
             float a = 0.f;
@@ -448,21 +455,37 @@ __global__ void __launch_bounds__(256) spmm_scalar_kernel(const SpmmProblem P) {
                 a = coef<EL>(P, base + lane, c);
             }
             const int cnt = (int)min((int64_t)32, p1 - base);
-            for (int j = 0; j < cnt; ++j) {
+            int j = 0;
+            for (; U > 1 && j + U <= cnt; j += U) {
+                uint32_t raw[U][T];
+                float aj[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int cj = __shfl_sync(FULL, c, j + u);
+                    aj[u] = __shfl_sync(FULL, a, j + u);
+                    const ST *r = B + (int64_t)cj * P.ldb + c0;
+#pragma unroll
+                    for (int t = 0; t < T; ++t) raw[u][t] = c0 + 32 * t < P.N ? ld_word(r + 32 * t) : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int t = 0; t < T; ++t)
+                        if (c0 + 32 * t < P.N) acc[t] = fmaf(aj[u], word_value<EL>(raw[u][t]), acc[t]);
+            }
+#pragma unroll 4
+            for (; j < cnt; ++j) {
                 const int cj = __shfl_sync(FULL, c, j);
                 const float aj = __shfl_sync(FULL, a, j);
+                const ST *r = B + (int64_t)cj * P.ldb + c0;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int col = c0 + lane + 32 * t;
-                    if (col < P.N) acc[t] = fmaf(aj, EL::scalar(B + (int64_t)cj * P.ldb + col), acc[t]);
-                }
+                for (int t = 0; t < T; ++t)
+                    if (c0 + 32 * t < P.N) acc[t] = fmaf(aj, EL::scalar(r + 32 * t), acc[t]);
             }
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int col = c0 + lane + 32 * t;
-            if (col < P.N) P.C[(int64_t)row * P.ldc + col] = acc[t] * sc;
-        }
+        for (int t = 0; t < T; ++t)
+            if (c0 + 32 * t < P.N) P.C[(int64_t)row * P.ldc + c0 + 32 * t] = acc[t] * sc;
     }
 }
 

@@ -66,3 +66,19 @@ def test_units_leave_infinities_where_they_are(gb):
     clean = A.colidx != 5
     B[5, 0] = 0
     assert np.array_equal(out[clean].astype(np.float64), oracle.sddmm(A.rowptr, A.colidx, vals, X, B)[0][clean])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "e4m3"])
+@pytest.mark.parametrize("N,base", [(24, 0), (66, 1), (96, 1), (97, 0), (120, 0), (127, 0), (128, 1), (161, 0)])
+def test_spmm_elements_bit_exact(gb, dtype, N, base):
+    """Single elements: three and four columns a lane, one and four entries in flight, whole and cut passes; units
+    halved so that half of the lanes have one (N = 24, 120)."""
+    import torch
+
+    A = gen.csr_from_lengths(LENGTHS, 1600, seed=815)
+    vals, B = gen.vals_int(A.nnz, 816, -4, 4), gen.dense_int(1600, N, 817, -4, 4)
+    one = lambda n: torch.ones(n, device="cuda") if dtype == "e4m3" else None
+    a = dev(oracle.e4m3_round(vals)) if dtype == "e4m3" else dev(vals).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    C = gb.spmm(dev(A.rowptr), dev(A.colidx), a, stored(B, dtype, base, N), a_scale=one(A.M), b_scale=one(1600),
+                variant="scalar")
+    assert np.array_equal(C.cpu().numpy().astype(np.float64), oracle.spmm(A.rowptr, A.colidx, vals, B)[0])
