@@ -1,4 +1,6 @@
 // SDDMM launches for every element type of X and Y.
+#include <math.h>
+
 #include "sddmm_kernels.cuh"
 
 namespace gbsp {
@@ -82,7 +84,15 @@ int launch_sddmm_typed(const SddmmProblem &P, int variant, int vecs, cudaStream_
         constexpr int ES = (int)sizeof(typename EL::stored);
         const int lx = unit_bytes(P.X, P.ldx, P.Kd, ES), ly = unit_bytes(P.Y, P.ldy, P.Kd, ES), lb = lx < ly ? lx : ly;
         const int units = P.Kd * ES / lb;
-        if (units >= 8 && units <= 256) {
+        // A row's start (X_i to registers) is most of the units' time on rows of a few entries and narrow Kd: 300,000 x
+        // 41,017, 2 entries a row, FP32 Kd = 9 / 21: 117 / 119 us, one lane per entry 48 / 72 (Zipf rows 56 / 58, 34 /
+        // 51); 200,000 x 3,000, 6 entries, 9 / 17: 82 / 84, 38 / 55.  With E4M3 units of 4 and 8 elements, all
+        // decoded for X_i, up to wider rows (6 entries, Kd = 72: 282, 212).  The lines lie where skewed rows, which a
+        // warp per row serves badly, are still served as fast (100,000 x 41,017, 6 entries, Zipf, FP32 13 / 17: 40 /
+        // 42 us, 35 / 50); even rows would do better with one lane per entry up to n Kd^2.5 = 26,500.
+        const double few = 5300.0 * (ES > 1 || lb < 4 ? 1 : lb < 8 ? 10 : 60);
+        const bool brief = P.nnz >= 0 && P.nnz < 8LL * P.M && pow((double)P.Kd, 2.5) * (double)P.nnz < few * (double)P.M;
+        if (units >= 8 && units <= 256 && !brief) {
             if constexpr (ES <= 1)
                 if (lb == 1) return run_units<EL, 1>(P, units, s);
             if constexpr (ES <= 2)

@@ -443,8 +443,9 @@ __global__ void __launch_bounds__(256) sddmm_unit_kernel(const SddmmProblem P, i
     }
 }
 
-// Any Kd and alignment (narrow ones, and those past the kernel above): one lane per stored entry, plain loads.  X_i is read by all lanes
-// of the warp at the same address (a broadcast).  Suits small Kd such as the paper's D = 2.
+// Any Kd and alignment (short rows of narrow ones, and those past the kernel above): one lane per stored entry,
+// plain loads.  X_i is read by all lanes of the warp at the same address (a broadcast).  Suits small Kd such
+// as the paper's D = 2.
 template <class EL>
 __global__ void __launch_bounds__(256) sddmm_scalar_kernel(const SddmmProblem P) {
     const int lane = threadIdx.x & 31;

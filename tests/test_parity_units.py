@@ -82,3 +82,18 @@ def test_spmm_elements_bit_exact(gb, dtype, N, base):
     C = gb.spmm(dev(A.rowptr), dev(A.colidx), a, stored(B, dtype, base, N), a_scale=one(A.M), b_scale=one(1600),
                 variant="scalar")
     assert np.array_equal(C.cpu().numpy().astype(np.float64), oracle.spmm(A.rowptr, A.colidx, vals, B)[0])
+
+
+@pytest.mark.parametrize("dtype,Kd", [("f32", 17), ("f32", 22), ("bf16", 33), ("e4m3", 36), ("e4m3", 72), ("e4m3", 104)])
+def test_sddmm_short_rows_bit_exact(gb, dtype, Kd):
+    """Rows of one to five entries on either side of the line between one lane per entry and the units."""
+    import torch
+
+    for mean in (2, 5):
+        A = gen.csr_from_lengths(np.tile(np.arange(2 * mean + 1), 300), 900, seed=820)
+        vals = gen.vals_int(A.nnz, 821, -4, 4)
+        X, Y = gen.dense_int(A.M, Kd, 822, -4, 4), gen.dense_int(A.K, Kd, 823, -4, 4)
+        one = lambda n: torch.ones(n, device="cuda") if dtype == "e4m3" else None
+        out = gb.sddmm(dev(A.rowptr), dev(A.colidx), dev(vals), stored(X, dtype, 0, Kd), stored(Y, dtype, 0, Kd),
+                       x_scale=one(A.M), y_scale=one(A.K), variant="scalar")
+        assert np.array_equal(out.cpu().numpy().astype(np.float64), oracle.sddmm(A.rowptr, A.colidx, vals, X, Y)[0])
