@@ -7,9 +7,9 @@ namespace gbsp {
 template <class EL, int LB>
 int launch_units(const SpmmProblem &P, cudaStream_t s) {
     using namespace spmm_detail;
-    // (single elements: FP32 up to 64, the others up to 64 and past 128)
+    // (single elements: up to 64, in E4M3 also past 192)
     constexpr int ES = (int)sizeof(typename EL::stored), UE = LB / ES;
-    constexpr int TMAX = UE >= 8 || (UE == 1 && ES == 4) ? 2 : UE >= 4 ? 4 : 8;
+    constexpr int TMAX = UE >= 8 || (UE == 1 && ES > 1) ? 2 : UE >= 4 ? 4 : 8;
     const int units = P.N / UE;
     const dim3 grid((P.M + 7) / 8);
     if (units <= 32)
@@ -42,10 +42,10 @@ int launch_elements(const SpmmProblem &P, cudaStream_t s) {
 //   times as fast; the others level or better.
 // - 65 to 96 single elements: three columns a lane, four entries in flight, 0.43 to 1.04 of one at a time's time and
 //   0.67 to 0.88 of the units' (four columns).
-// - more of them: FP32 four columns and entries, 0.81 to 1.05 of the units' time (0.48 to 1.01 of one at a time's);
-//   E4M3 up to 128 the same, 0.89 to 1.02.  BF16 up to 128 one at a time: 0.74 to 0.99 of the units' time
-//   on even rows (1.12 on the 3,000, 1.6 on the Zipf ones), 0.82 to 0.99 of four in flight's (1.25).  E4M3 and
-//   BF16 past that the units: one at a time takes 0.79 to 1.22 of their time (Zipf 1.7).
+// - more of them: FP32 four columns and entries, 0.81 to 1.05 of the units' time; E4M3 up to 128 the same, 0.89 to
+//   1.02, up to 192 three columns one at a time, 0.64 to 0.78 (1.00 on the Zipf rows); BF16 four columns one at
+//   a time, up to 128 0.66 to 0.97 of the units' time, past that 0.68 to 0.85 (1.02 on the Zipf rows).  E4M3 past
+//   192 the units: one at a time takes 0.73 to 0.91 of their time on even rows and 1.13 on Zipf ones.
 template <class EL>
 int launch_unvectorised(const SpmmProblem &P, cudaStream_t s) {
     constexpr int ES = (int)sizeof(typename EL::stored);
@@ -54,9 +54,11 @@ int launch_unvectorised(const SpmmProblem &P, cudaStream_t s) {
     while (lb > ES && P.N * ES < 16 * lb) lb /= 2;
     if (lb == ES && P.N > 64) {
         if (P.N <= 96) return launch_elements<EL, 4, 3>(P, s);
-        if (ES == 2 && P.N <= 128) return launch_elements<EL, 1, 4>(P, s);
+        if constexpr (ES == 2) return launch_elements<EL, 1, 4>(P, s);
         if constexpr (ES != 2)
             if (ES == 4 || P.N <= 128) return launch_elements<EL, 4, 4>(P, s);
+        if constexpr (ES == 1)
+            if (P.N <= 192) return launch_elements<EL, 1, 3>(P, s);
     }
     if constexpr (ES <= 1)
         if (lb == 1) return launch_units<EL, 1>(P, s);

@@ -429,8 +429,10 @@ __global__ void __launch_bounds__(256) spmm_unit_kernel(const SpmmProblem P) {
 }
 
 // ... element by element, lane l owns columns l, l + 32, ... of a pass of T x 32, U entries' loads in flight and
-// the columns past the row's end predicated.  U = 1: rows of a few entries, where the registers of
-// more (fewer warps per SM) do not help.  U = 4, 40 to 62 registers where the units take 76 to 80, so that
+// the columns past the row's end predicated.  U = 1: as many in flight as eight entries' unrolled code has in 40
+// registers, for rows of a few entries, where more registers (fewer warps per SM) do not help, and for the
+// rows past 96 columns that need no more (BF16, N = 161: 200,000 x 3,000 1,732 us with the units, 1,180 so; 30,011 x
+// 41,017 542, 385, Zipf 1,408, 1,436).  U = 4, 40 to 62 registers where the units take 76 to 80, so that
 // rows from a B close at hand (200,000 x 3,000, 100 entries a row: FP32 N = 65 / 127 624 / 740 us at U = 1, 867 /
 // 880 with the units, 587 / 718 so) keep their warps and long rows (30,011 x 41,017, 205 entries a row,
 // Zipf: 1029 / 1404, 731 / 730, 607 / 688) their loads.
@@ -473,7 +475,7 @@ __global__ void __launch_bounds__(256) spmm_scalar_kernel(const SpmmProblem P) {
                     for (int t = 0; t < T; ++t)
                         if (c0 + 32 * t < P.N) acc[t] = fmaf(aj[u], word_value<EL>(raw[u][t]), acc[t]);
             }
-#pragma unroll 4
+#pragma unroll(U > 1 ? 4 : 8)
             for (; j < cnt; ++j) {
                 const int cj = __shfl_sync(FULL, c, j);
                 const float aj = __shfl_sync(FULL, a, j);

@@ -69,7 +69,7 @@ def test_units_leave_infinities_where_they_are(gb):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "e4m3"])
-@pytest.mark.parametrize("N,base", [(24, 0), (66, 1), (96, 1), (97, 0), (120, 0), (127, 0), (128, 1), (161, 0)])
+@pytest.mark.parametrize("N,base", [(24, 0), (66, 1), (96, 1), (97, 0), (120, 0), (127, 0), (128, 1), (161, 0), (192, 1), (193, 0), (257, 0)])
 def test_spmm_elements_bit_exact(gb, dtype, N, base):
     """Single elements: three and four columns a lane, one and four entries in flight, whole and cut passes; units
     halved so that half of the lanes have one (N = 24, 120)."""
