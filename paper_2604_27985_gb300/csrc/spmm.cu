@@ -35,17 +35,18 @@ int launch_elements(const SpmmProblem &P, cudaStream_t s) {
 
 // The unvectorised kernels, by what the rows' alignment allows (lb bytes a load) and what was measured on 30,011
 // x 41,017 (20 and 205 entries a row, even and Zipf), 4,000 x 41,017 (1,500), 200,000 x 3,000 (100), 3,000 x 3,000
-// (200) and 20,000 x 250,000 (60, clustered), times of the first of two over the second:
+// (200) and 20,000 x 250,000 (60, clustered):
 // - rows averaging under 16 entries (or not said): one entry at a time.  200,000 x 3,000, 6 entries a row,
 //   N = 101: 85 us against 117 for the units.
 // - wide loads that leave half of the lanes without one are halved: E4M3 N = 24 to 120 from 8 bytes 1.4 to 2.8
 //   times as fast; the others level or better.
-// - 65 to 96 single elements: three columns a lane, four entries in flight, 0.43 to 1.04 of one at a time's time and
-//   0.67 to 0.88 of the units' (four columns).
+// - 65 to 96 single elements: three columns a lane, four entries in flight, 0.67 to 0.88 of the units' time (four
+//   columns), 0.82 to 1.10 of one at a time's (the lower end on Zipf rows).
 // - more of them: FP32 four columns and entries, 0.81 to 1.05 of the units' time; E4M3 up to 128 the same, 0.89 to
-//   1.02, up to 192 three columns one at a time, 0.64 to 0.78 (1.00 on the Zipf rows); BF16 four columns one at
-//   a time, up to 128 0.66 to 0.97 of the units' time, past that 0.68 to 0.85 (1.02 on the Zipf rows).  E4M3 past
-//   192 the units: one at a time takes 0.73 to 0.91 of their time on even rows and 1.13 on Zipf ones.
+//   1.02 (one at a time takes 0.78 to 0.99 of theirs on even rows, 1.03 to 1.07 on Zipf ones).  E4M3 up to 192
+//   three columns one at a time, 0.64 to 0.89 of the units' time; BF16 four columns one at a time, up to 128 0.66
+//   to 0.98, past that 0.68 to 0.85 (1.02 on Zipf rows).  E4M3 past 192 the units: one at a time takes 0.73 to 0.91
+//   of their time on even rows and 1.13 on Zipf ones.
 template <class EL>
 int launch_unvectorised(const SpmmProblem &P, cudaStream_t s) {
     constexpr int ES = (int)sizeof(typename EL::stored);

@@ -339,10 +339,9 @@ __global__ void __launch_bounds__(256) spmm_rowgroup_kernel(const SpmmProblem P)
 // Any width and alignment: one warp per row, loads of LB bytes (as many whole elements as the
 // rows' alignment and width allow, UE of them), lane l owns units l, l + 32, ... of a pass of T x 32
 // units.  U entries' units are loaded before any is used and the next 32 entries while these are
-// worked on; bound by the latency of both.  30,011 x 41,017, 205 entries a row, FP32: N = 110 321 ->
-// 190 us, 101 321 -> 278, 9 221 -> 119 (the form below); Zipf rows, N = 101: 1403 -> 730.  Twice or half
-// the entries in flight: 287 / 291 at N = 101.  Each column is summed entry by entry in order,
-// whatever T, U and LB are.
+// worked on; bound by the latency of both.  30,011 x 41,017, 205 entries a row, FP32: N = 110 321 -> 190 us,
+// 9 221 -> 119 (the form below, one entry at a time).  Each column is summed entry by entry in order, whatever
+// T, U and LB are.
 template <class EL, int LB, int T>
 __global__ void __launch_bounds__(256) spmm_unit_kernel(const SpmmProblem P) {
     constexpr int UE = LB / (int)sizeof(typename EL::stored);
@@ -428,14 +427,12 @@ __global__ void __launch_bounds__(256) spmm_unit_kernel(const SpmmProblem P) {
     }
 }
 
-// ... element by element, lane l owns columns l, l + 32, ... of a pass of T x 32, U entries' loads in flight and
-// the columns past the row's end predicated.  U = 1: as many in flight as eight entries' unrolled code has in 40
-// registers, for rows of a few entries, where more registers (fewer warps per SM) do not help, and for the
-// rows past 96 columns that need no more (BF16, N = 161: 200,000 x 3,000 1,732 us with the units, 1,180 so; 30,011 x
-// 41,017 542, 385, Zipf 1,408, 1,436).  U = 4, 40 to 62 registers where the units take 76 to 80, so that
-// rows from a B close at hand (200,000 x 3,000, 100 entries a row: FP32 N = 65 / 127 624 / 740 us at U = 1, 867 /
-// 880 with the units, 587 / 718 so) keep their warps and long rows (30,011 x 41,017, 205 entries a row,
-// Zipf: 1029 / 1404, 731 / 730, 607 / 688) their loads.
+// ... element by element, lane l owns columns l, l + 32, ... of a pass of T x 32, the columns past the row's end
+// predicated.  U = 1: eight entries' code unrolled in 40 registers (the units take 76 to 80, and so fewer warps per
+// SM), for rows of a few entries and for rows past 96 columns.  U = 4: four entries' loads before their sums, 48 to
+// 63 registers, for long rows that others wait for.  Times in us of the units, U = 1, U = 4, on 200,000 x 3,000 (100
+// entries a row, B close at hand) and 30,011 x 41,017 (205 entries a row, Zipf): FP32 N = 65 870, 537, 590 and
+// 731, 691, 606; N = 127 882, 590, 719 and 735, 713, 688; BF16 N = 161 1,732, 1,182 and 1,408, 1,427 (U = 1).
 template <class EL, int U, int T>
 __global__ void __launch_bounds__(256) spmm_scalar_kernel(const SpmmProblem P) {
     using ST = typename EL::stored;

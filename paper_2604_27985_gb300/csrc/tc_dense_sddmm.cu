@@ -15,7 +15,7 @@
 //
 // 16,384^2 at 90%, half in dense blocks, Kd = 256: BF16 on a plan 637 -> 215 us, where the MMAs alone
 // (N = 64 reads A's rows from shared memory for little work: 92 clocks each) take 152; E4M3 without
-// a plan 804 -> 447 with the regrouping's 130.  On the way: 328 us with the tile coordinates by
+// a plan 804 -> 446 with the regrouping's 172 (260 here: fewer MMA steps, more instructions per entry).  On the way: 328 us with the tile coordinates by
 // 64-bit division in every warp, 245 without.
 #include <mutex>
 
@@ -426,7 +426,8 @@ bool sddmm_pays(int64_t M, int64_t K, int64_t Kd, int64_t nnz, bool fp8) {
 }
 
 // ... with the regrouping in every call (0.6 ns per entry of a block of rows, a wave of blocks at a
-// time).  E4M3 only: at Kd <= 256 its error is below the CSR kernel's (3.0e-8 against 4.55e-8 on
+// time; 0.8 with the positions on 16,384^2, where at Kd = 128 the two paths take the same time and whole
+// tiles are the more exact one).  E4M3 only: at Kd <= 256 its error is below the CSR kernel's (3.0e-8 against 4.55e-8 on
 // 16,384^2 at 90%, Kd = 256), BF16's four steps per part have the larger one
 // (8.0e-8 against 6.1e-8).  The E4M3 CSR kernel is bound by its conversions: 16 / 30 ps per entry at
 // Kd = 128 / 256.  Where the scratch passes the pool's limit (from 134 million entries on) a tile was measured at

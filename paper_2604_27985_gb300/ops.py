@@ -205,6 +205,8 @@ def launch_count() -> int:
 class TcPlan:
     """Condensed-tile tensor-core plan of a BF16 or per-row-scaled E4M3 CSR matrix
     (gbsp_plan_create): dense 16 x 8 blocks run on tcgen05, the rest on the CSR kernels.
+    With the default threshold and residual kernel, executions take whole 128 x 64 tiles
+    instead where that is faster and no less exact (``info`` describes the blocks).
     ``execute(B)`` returns C = A B (E4M3: ``execute(B, row_scale=t)``)."""
 
     def __init__(self, rowptr, colidx, vals, ncols, threshold=0, *, row_scale=None, residual_variant="auto",
@@ -227,7 +229,8 @@ class TcPlan:
     def sddmm(self, svals, X, Y, out=None, x_scale=None, y_scale=None, tiles=-1, stream=None) -> torch.Tensor:
         """out[p] = svals[p] <X_i, Y_j> on the plan's pattern (gbsp_plan_sddmm): the dense
         blocks on tcgen05 and the rest on the CSR kernel (tiles=1), every entry on the CSR
-        kernels (tiles=0), or the plan's choice (tiles=-1); returns FP32 out[nnz]."""
+        kernels (tiles=0), or the plan's choice (tiles=-1; also whole tiles); returns FP32
+        out[nnz]."""
         if out is None:
             out = torch.empty(svals.numel(), dtype=torch.float32, device=X.device)
         x, y = _dense(X, x_scale), _dense(Y, y_scale)
