@@ -269,7 +269,8 @@ __device__ __forceinline__ void st_shared_zero16(uint32_t addr) {
 // dense blocks, N = 256 (the 16 x 8 blocks + residual kernel before: 415 us): 264 us with two
 // groups and entries loaded to registers a tile ahead, 170 with the entries copied to shared
 // memory, 150 with four groups, 124 with the entry loop unpredicated, 119 with the MMAs issued
-// from a uniform loop.
+// from a uniform loop, 116 with an accumulator's tiles a constant of that loop.  (Accumulators ended tile by tile,
+// by entries counted in the kernel: 143, in the loop's branches.)
 template <int NT>
 __global__ void __launch_bounds__(kThreads, 1) spmm_kernel(const __grid_constant__ CUtensorMap tmB,
                                                                          const Args a) {
