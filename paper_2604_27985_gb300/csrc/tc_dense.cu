@@ -642,17 +642,29 @@ static bool sums_as_well(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 // The plan's blocks and CSR residual take 6.8 / 9.0 / 15.9 ps per entry at 64 / 128 / 256 features
 // where they do best (clustered, 5%), more on unstructured rows (11 / 13 / 20).  On 16,384^2 the
 // lines cross near 6.5% / 5% / 3% of entries.
-// Its blocks' MMAs run one accumulator over all of a row's entries in blocks, the share s of them, and so lose
+static bool faster(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+    if (M < 2048 || K < 2048 || N < 64 || N > 512 || (double)nnz < 0.03 * (double)M * (double)K) return false;
+    int64_t waves;
+    return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+}
+
+// The blocks' MMAs run one accumulator over all of a row's entries in blocks, the share s of them, and so lose
 // about s^2 K / 512 times what whole tiles do: at 512 the errors are level (2,048 columns, half in
 // blocks: 1.00 at 2.5% of entries, 0.79 at 10%), above that whole tiles have the smaller one (0.13 of it
 // on 16,384 columns at 10%), below it only where their sums are as exact as the CSR kernels', which
 // then have most of the entries (8% of 3,072 columns, a fifth in blocks: 6.2e-8 against 7.3e-8 at 64 features).
-bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz) {
-    if (M < 2048 || K < 2048 || N < 64 || N > 512 || (double)nnz < 0.03 * (double)M * (double)K) return false;
+static bool no_less_exact(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz) {
     const double share = (double)dense_nnz / (double)nnz;
-    if ((double)K * share * share < kChunk * kCols && !sums_as_well(M, K, N, nnz)) return false;
-    int64_t waves;
-    return product_us(M, K, N, &waves) < 0.9e-6 * (double)nnz * (2.5 + 0.05 * (double)N);
+    return (double)K * share * share >= kChunk * kCols || sums_as_well(M, K, N, nnz);
+}
+
+bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz) {
+    return faster(M, K, N, nnz) && no_less_exact(M, K, N, nnz, dense_nnz);
+}
+
+bool spmm_may_pay(int64_t M, int64_t K, int64_t nnz, int64_t dense_nnz) {
+    return faster(M, K, 256, nnz) &&
+           (no_less_exact(M, K, 256, nnz, dense_nnz) || no_less_exact(M, K, 512, nnz, dense_nnz));
 }
 
 // For rows of even length (the split AUTO would take is the row split).  The regrouping takes 0.5 ns

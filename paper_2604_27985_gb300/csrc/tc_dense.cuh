@@ -40,6 +40,8 @@ inline double scratch_us(int64_t bytes) {
 bool tiles_fit(int64_t M, int64_t K, int64_t nnz);
 // (dense_nnz: the entries that a plan's 16 x 8 blocks would hold)
 bool spmm_pays(int64_t M, int64_t K, int64_t N, int64_t nnz, int64_t dense_nnz);
+// ... for a plan, whose N is not known yet: at 256 features, in accuracy at 512 if not.
+bool spmm_may_pay(int64_t M, int64_t K, int64_t nnz, int64_t dense_nnz);
 // ... also where the regrouping is part of every call, against the CSR kernels.
 bool spmm_pays_unplanned(int64_t M, int64_t K, int64_t N, int64_t nnz);
 

@@ -881,9 +881,7 @@ GBSP_EXPORT int gbsp_plan_create(const gbsp_csr *A, int32_t threshold, const gbs
     // the plan: at a few percent of entries and more, whole tiles on the tensor cores
     // (an E4M3 plan's SpMM does not take them, its SDDMM past Kd = 256 where the tiles do)
     if (by_default && dense::tiles_fit(M, K, p->nnz) &&
-        ((!fp8 && (dense::spmm_pays(M, K, 256, p->nnz, p->dense_nnz) ||
-                   dense::spmm_pays(M, K, 512, p->nnz, p->dense_nnz))) ||
-         dense::sddmm_pays(M, K, 256, p->nnz, fp8) ||
+        ((!fp8 && dense::spmm_may_pay(M, K, p->nnz, p->dense_nnz)) || dense::sddmm_pays(M, K, 256, p->nnz, fp8) ||
          (fp8 && takes_tiles(p) && dense::sddmm_pays(M, K, dense::sddmm_max_kd(fp8), p->nnz, fp8)))) {
         if (dev_alloc(&p->tiles.ent, (size_t)dense::ent_count(p->nnz)) == GBSP_OK &&
             dev_alloc(&p->tiles.tptr, (size_t)(dense::row_blocks(M) * (dense::col_tiles(K) + 1))) == GBSP_OK &&
